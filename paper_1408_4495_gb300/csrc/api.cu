@@ -987,7 +987,8 @@ ls_status ls_far_field(ls_ctx* c, int nrhs, const double* dirs, const double* us
     copy_in(c, dd, dirs, (size_t)nrhs * c->d * sizeof(double));
     copy_in(c, od, obs, (size_t)nobs * c->d * sizeof(double));
     copy_in(c, ud, us, tot * sizeof(double2));
-    ls::far_field(c->d, c->n, nrhs, nobs, ud, dd, od, c->w2m64, c->omega, c->h, fd, c->st);
+    double2* scratch = buf<double2>(c, "ff_scratch", ls::far_scratch_elems(c->d, c->n, nrhs, nobs));
+    ls::far_field(c->d, c->n, nrhs, nobs, ud, dd, od, c->w2m64, c->omega, c->h, fd, scratch, c->st);
     copy_out(c, out, fd, (size_t)nrhs * nobs * sizeof(double2));
     LS_CUDA(cudaStreamSynchronize(c->st));
     return LS_OK;

@@ -94,7 +94,8 @@ void build_kernel_table(int d, int n, double omega, double h, double2* ktq, cuda
 // far-field pattern u_inf(theta_k; r) of the scattered fields us (nrhs x N) of the plane waves
 // dirs (nrhs x d) in the directions obs (nobs x d); out: nrhs x nobs
 void far_field(int d, int n, int nrhs, int nobs, const double2* us, const double* dirs, const double* obs,
-               const double* w, double omega, double h, double2* out, cudaStream_t st);
+               const double* w, double omega, double h, double2* out, double2* scratch, cudaStream_t st);
+size_t far_scratch_elems(int d, int n, int nrhs, int nobs);  // scratch: tables and partial sums
 void point_source(int d, int n, int nrhs, const int* pts, const double2* q, const double2* ktq, double h, double2* g,
                   cudaStream_t st);
 void build_symbol(const ConvPlan& p, const double2* ktq, double2* sym64, float2* sym32, double2* work,

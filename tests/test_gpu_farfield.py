@@ -90,3 +90,25 @@ def test_far_field_refused_for_laplace(LS):
         with pytest.raises(LS.LsError) as e:
             s.far_field(np.array([[1.0, 0, 0]]), np.zeros((1, 16, 16, 16), complex), np.array([[1.0, 0, 0]]))
         assert e.value.status == LS.LS_ESTATE
+
+
+@pytest.mark.parametrize("d,n,nrhs,nobs", [(2, 16, 1, 1), (2, 24, 2, 17), (2, 48, 1, 33), (2, 256, 2, 65), (2, 64, 1, 9000),
+                                           (3, 8, 1, 16), (3, 24, 2, 31)])
+def test_far_field_tile_edges(LS, d, n, nrhs, nobs):
+    """Line tiles with a remainder, every direction tile (16, 32, 64) with idle columns, a second
+    tile, and fields that are not finite where the medium vanishes (those points do not enter).
+    FP64 sums of at most n^d terms against the oracle's: the bound of the tests above."""
+    omega = 2 * math.pi * n / 8
+    m = medium(d, n, 4)
+    dirs, obs = obs_dirs(d, nrhs, 9), obs_dirs(d, nobs, 5)
+    rng = np.random.default_rng(1)
+    us = rng.standard_normal((nrhs,) + (n,) * d) + 1j * rng.standard_normal((nrhs,) + (n,) * d)
+    dirty = us.copy()
+    dirty[:, m == 0.0] = np.nan
+    with LS.Solver(m, omega, mixed=True) as s:
+        F = s.far_field(dirs, dirty, obs)
+    pick = range(0, nobs, max(1, nobs // 70))
+    for r in range(nrhs):
+        ut = O.plane_wave(n, d, omega, dirs[r]) + us[r]
+        ref = O.far_field(n, d, omega, m, ut, obs[list(pick)])
+        assert np.max(np.abs(F[r][list(pick)] - ref)) < 1e-12 * np.max(np.abs(ref))
