@@ -120,6 +120,27 @@ struct StencilKey {
 };
 std::map<StencilKey, std::pair<std::vector<double2>, std::vector<double2>>> g_stencil_cache;
 
+// host twiddle tables per FFT length (one of eleven), kept for the process
+struct LineTables {
+  std::vector<double2> t64, sym;  // the passes' (16-byte values), the symbol transforms'
+  std::vector<float2> t32;        // the FP32 passes'
+};
+const LineTables& line_tables(int L) {
+  static std::mutex mu;
+  static std::map<int, LineTables> cache;
+  std::lock_guard<std::mutex> lk(mu);
+  LineTables& t = cache[L];  // (map nodes stay where they are)
+  if (t.t32.empty()) {
+    ls::line_twiddles(L, true, t.t64);
+    ls::symbol_twiddles(L, t.sym);
+    std::vector<double2> tp;
+    ls::line_twiddles(L, false, tp);
+    t.t32.resize(tp.size());
+    for (size_t q = 0; q < tp.size(); ++q) t.t32[q] = make_float2((float)tp[q].x, (float)tp[q].y);
+  }
+  return t;
+}
+
 bool is_device_ptr(const void* p) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -258,7 +279,7 @@ template <typename C> void op_apply(ls_ctx* c, int nrhs, const C* u, C* y) {
   const size_t s1 = ls::conv_scratch1_elems(c->d, c->n, nrhs), s2 = ls::conv_scratch2_elems(c->d, c->n, nrhs);
   void* t1 = buf<C>(c, sizeof(C) == 8 ? "conv1_32" : "conv1_64", s1);
   void* t2 = s2 ? buf<C>(c, sizeof(C) == 8 ? "conv2_32" : "conv2_64", s2) : nullptr;
-  ls::conv_apply<C>(c->plan, nrhs, u, y, nullptr, true, t1, t2, c->st);
+  ls::conv_apply<C>(c->plan, nrhs, u, y, t1, t2, c->st);
 }
 
 // y = (I + K omega^2 m) u, or y = sub - (I + K omega^2 m) u, in float-float arithmetic
@@ -760,21 +781,14 @@ static ls_status setup_common(const ls_grid* g, double omega, const double* m, b
     c->w2m32 = dalloc<float>(c->N);
     LS_CUDA(cudaMemcpyAsync(c->w2m64, w64.data(), c->N * sizeof(double), cudaMemcpyHostToDevice, c->st));
     LS_CUDA(cudaMemcpyAsync(c->w2m32, w32.data(), c->N * sizeof(float), cudaMemcpyHostToDevice, c->st));
-    // twiddles: exp(-2 pi i m / L) for the FP64 and float-float passes, the per-pass table of
-    // the FP32 passes (fft_plan.h)
+    // twiddle tables of the passes: FP32 (8-byte values), FP64 and float-float (16-byte values)
     const int L = c->L;
-    std::vector<double2> t64(L), tp;
-    for (int q = 0; q < L; ++q) {
-      const double a = -2.0 * M_PI * (double)q / (double)L;
-      t64[q] = make_double2(std::cos(a), std::sin(a));
-    }
-    ls::fft_twiddles(L, tp);
-    std::vector<float2> t32(tp.size());
-    for (size_t q = 0; q < tp.size(); ++q) t32[q] = make_float2((float)tp[q].x, (float)tp[q].y);
-    c->tw64 = dalloc<double2>(L);
-    c->tw32 = dalloc<float2>(t32.size());
-    LS_CUDA(cudaMemcpyAsync(c->tw64, t64.data(), L * sizeof(double2), cudaMemcpyHostToDevice, c->st));
-    LS_CUDA(cudaMemcpyAsync(c->tw32, t32.data(), t32.size() * sizeof(float2), cudaMemcpyHostToDevice, c->st));
+    const LineTables& tab = line_tables(L);
+    const std::vector<double2>&t64 = tab.t64, &ts = tab.sym;
+    c->tw64 = dalloc<double2>(t64.size());
+    c->tw32 = dalloc<float2>(tab.t32.size());
+    LS_CUDA(cudaMemcpyAsync(c->tw64, t64.data(), t64.size() * sizeof(double2), cudaMemcpyHostToDevice, c->st));
+    LS_CUDA(cudaMemcpyAsync(c->tw32, tab.t32.data(), tab.t32.size() * sizeof(float2), cudaMemcpyHostToDevice, c->st));
     // Nystrom table quadrant and symbol (Sec. 2.1)
     const long n1 = n + 1;
     const long nq = c->d == 2 ? n1 * n1 : n1 * n1 * n1;
@@ -800,9 +814,10 @@ static ls_status setup_common(const ls_grid* g, double omega, const double* m, b
     c->plan.w2m64 = c->w2m64;
     {
       const long Ld = c->d == 2 ? (long)L * L : (long)L * L * L;
-      double2* work = dalloc<double2>(Ld);
+      double2* work = dalloc<double2>(Ld + ts.size());  // the transform, then its twiddle table
       try {
-        ls::build_symbol(c->plan, c->ktq, c->sym64, c->sym32, work, c->st);
+        LS_CUDA(cudaMemcpyAsync(work + Ld, ts.data(), ts.size() * sizeof(double2), cudaMemcpyHostToDevice, c->st));
+        ls::build_symbol(c->d, n, c->ktq, c->sym64, c->sym32, work, work + Ld, c->st);
         LS_CUDA(cudaStreamSynchronize(c->st));
       } catch (...) {
         ls::dev_free(work);
@@ -813,10 +828,10 @@ static ls_status setup_common(const ls_grid* g, double omega, const double* m, b
     c->plan.sym32 = c->sym32;
     c->plan.sym64 = c->sym64;
     {
-      const size_t ntwf = 2 * (size_t)L, nsy = 2 * (size_t)nq;  // FP64 components: one float pair each
+      const size_t ntwf = 2 * t64.size(), nsy = 2 * (size_t)nq;  // FP64 components: one float pair each
       c->ffbuf = dalloc<float2>(ntwf + nsy + (size_t)c->N);
-      ls::to_ff(reinterpret_cast<const double*>(c->tw64), c->ffbuf, (long)ntwf, c->st);
-      ls::to_ff(reinterpret_cast<const double*>(c->sym64), c->ffbuf + ntwf, (long)nsy, c->st);
+      ls::to_ffp(c->tw64, c->ffbuf, (long)t64.size(), c->st);
+      ls::to_ffp(c->sym64, c->ffbuf + ntwf, nq, c->st);
       ls::to_ff(c->w2m64, c->ffbuf + ntwf + nsy, c->N, c->st);
       c->plan.twff = c->ffbuf;
       c->plan.symff = c->ffbuf + ntwf;
@@ -931,9 +946,8 @@ ls_status ls_rhs_plane_wave(ls_ctx* c, int nrhs, const double* dirs, double* g_o
     }
     copy_in(c, dd, dirs, (size_t)nrhs * c->d * sizeof(double), st);
     // float-float passes on the mixed path, FP64 on the plain path
-    if (c->prec == LS_PREC_MIXED)
-      ls::conv_rhs_ff(c->plan, nrhs, dd, gd, t1, t2, buf<ffc>(c, "rhs_phase", (size_t)nrhs * c->d * c->n), st);
-    else ls::conv_apply<double2>(c->plan, nrhs, (const double2*)nullptr, gd, dd, false, t1, t2, st);
+    ls::conv_rhs(c->plan, nrhs, dd, gd, c->prec != LS_PREC_MIXED, t1, t2,
+                 buf<double2>(c, "rhs_phase", (size_t)nrhs * c->d * c->n), st);
     copy_out(c, g_out, gd, tot * sizeof(double2), st);
     LS_CUDA(cudaStreamSynchronize(st));
     return LS_OK;

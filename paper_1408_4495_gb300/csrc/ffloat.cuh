@@ -140,7 +140,7 @@ __device__ __forceinline__ double ff_to_f64(ff a) { return f64_of(a.hi) + f64_of
 __device__ __forceinline__ double2 ffc_to_f64(ffc v) { return make_double2(ff_to_f64(v.x), ff_to_f64(v.y)); }
 
 // an FP64 number as a float-float: hi = its leading 24 significant bits (truncated), lo =
-// the next 23 bits (truncated), so |x - (hi + lo)| < 2^-46 |x|; lo is built as an exact
+// the next 23 bits (rounded half up), so |x - (hi + lo)| <= 2^-47 |x|; lo is built as an exact
 // FP32 integer (the magic-number form) scaled by a power of two.  Outside
 // 2^-74 <= |x| < 2^128 (where lo or hi would leave the FP32 normal range) and for
 // infinities and NaNs the FP64 conversion is used; zeros stay zeros.  |lo| may reach
@@ -152,9 +152,10 @@ __device__ __forceinline__ ff ff_of_f64(double x) {
   if (e == 0u) return ff(__uint_as_float(sign), 0.f);
   if (e - 949u < 1150u - 949u + 1u) {
     const unsigned hi = sign | ((e - (1023u - 127u)) << 23) | (unsigned)((b >> 29) & 0x7fffffu);
-    const unsigned r = (unsigned)(b >> 6) & 0x7fffffu;  // fraction bits 28..6
-    // r as an FP32 integer: 2^23 + r has the exponent field of 2^23 and fraction r
-    const float rf = __fsub_rn(__uint_as_float(0x4b000000u | r), 8388608.0f);
+    const unsigned r = (((unsigned)(b >> 5) & 0xffffffu) + 1u) >> 1;  // fraction bits 28..6, rounded
+    // r <= 2^23 as an FP32 integer: 2^23 + r has the exponent field of 2^23 and fraction r (a
+    // carry into the exponent makes it 2^24)
+    const float rf = __fsub_rn(__uint_as_float(0x4b000000u + r), 8388608.0f);
     // lo = r * 2^(E - 46), E = e - 1023 the unbiased exponent of x
     const float scale = __uint_as_float((e - (1023u + 46u - 127u)) << 23);
     return ff(__uint_as_float(hi), __uint_as_float(__float_as_uint(__fmul_rn(rf, scale)) | sign));

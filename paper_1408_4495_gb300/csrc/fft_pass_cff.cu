@@ -4,11 +4,11 @@
 
 namespace ls {
 
-#define LS_DECL(LL) LS_PASS_INST(extern, ffc, LL)
+#define LS_DECL(LL) LS_PASS_INST(extern, ffp, LL)
 LS_FOR_L(LS_DECL)
 #undef LS_DECL
 
-template void row_pass<ffc>(int, int, const RowPassArgs&, cudaStream_t);
-template void col_pass<ffc>(int, int, const ColPassArgs&, cudaStream_t);
+template void row_pass<ffp>(int, int, const RowPassArgs&, cudaStream_t);
+template void col_pass<ffp>(int, int, const ColPassArgs&, cudaStream_t);
 
 }  // namespace ls

@@ -3,12 +3,12 @@
 
 namespace ls {
 
-LS_PASS_INST(, ffc, 16)
-LS_PASS_INST(, ffc, 32)
-LS_PASS_INST(, ffc, 48)
-LS_PASS_INST(, ffc, 64)
-LS_PASS_INST(, ffc, 96)
-LS_PASS_INST(, ffc, 128)
-LS_PASS_INST(, ffc, 256)
+LS_PASS_INST(, ffp, 16)
+LS_PASS_INST(, ffp, 32)
+LS_PASS_INST(, ffp, 48)
+LS_PASS_INST(, ffp, 64)
+LS_PASS_INST(, ffp, 96)
+LS_PASS_INST(, ffp, 128)
+LS_PASS_INST(, ffp, 256)
 
 }  // namespace ls

@@ -3,7 +3,7 @@
 
 namespace ls {
 
-LS_PASS_INST(, ffc, 512)
-LS_PASS_INST(, ffc, 1024)
+LS_PASS_INST(, ffp, 512)
+LS_PASS_INST(, ffp, 1024)
 
 }  // namespace ls

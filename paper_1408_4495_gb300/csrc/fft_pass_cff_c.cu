@@ -3,7 +3,7 @@
 
 namespace ls {
 
-LS_PASS_INST(, ffc, 2048)
-LS_PASS_INST(, ffc, 4096)
+LS_PASS_INST(, ffp, 2048)
+LS_PASS_INST(, ffp, 4096)
 
 }  // namespace ls

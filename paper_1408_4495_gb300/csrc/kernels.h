@@ -10,24 +10,19 @@ namespace ls {
 
 // ---------------------------------------------------------------- FFT passes (fft.cu)
 struct RowPassArgs {
-  const void* in;      // lines of complex (path precision), line stride in_ls
+  const void* in;      // lines of n (forward) or 2n (inverse) complex entries, line stride in_ls
   void* out;           // line stride out_ls
   long lines;
-  int n_in, n_out;     // entries read (zero padded to L) / entries written
   long in_ls, out_ls;
-  const void* pw;      // real weights [(line % pw_lines) * n_in + e], or null
+  const void* pw;      // forward: real weights [(line % pw_lines) * n + e]
   long pw_lines;
-  const void* tw;      // twiddles exp(-2 pi i m / L), m < L
-  const double* plane_dirs;  // right-hand-side prologue (FP64 and float-float passes), or null
-  const double* pw64;  // omega^2 m in FP64 for that prologue
-  const void* phase;   // float-float passes: the prologue's phase factors as float-float
-                       // complex [rhs][axis][k] = exp(i omega h (k + 1) dir_axis), or null
-  int d, n;
-  double omega, h;
-  const void* addv;    // epilogue: out += addv[line * add_ls + e], or null
+  const void* tw;      // twiddle table of the arithmetic (line_twiddles)
+  const void* phase;   // forward: per-axis phase factors of plane waves [rhs][axis][k] to
+                       // transform -pw exp(i omega x . dir) instead of in, or null
+  int d;
+  const void* addv;    // inverse: out += addv[line * add_ls + e], or null
   long add_ls;
-  const void* subv;    // epilogue: out = subv - (...), or null (float-float passes only)
-  int in64, out64;     // float-float passes: in / out, addv, subv are FP64 complex
+  const void* subv;    // inverse: out = subv - (...), or null (FP64 output only)
 };
 
 struct ColPassArgs {
@@ -35,16 +30,15 @@ struct ColPassArgs {
   void* out;
   long outer, inner;   // lines = outer * inner, inner index contiguous in memory
   long in_os, in_es, out_os, out_es;
-  int n_in, n_out;
   const void* sym;     // symbol quadrant (n+1)^d for the symbol pass
-  int n, d;
+  int d;
   const void* tw;
 };
 
 struct ConvPlan {
   int d, n;
   double omega, h;
-  const float2* tw32;
+  const float2* tw32;   // twiddle tables (line_twiddles) in FP32, FP64, float-float
   const double2* tw64;
   const float2* sym32;
   const double2* sym64;
@@ -58,16 +52,15 @@ struct ConvPlan {
 template <typename C> void row_pass(int L, int sign, const RowPassArgs& a, cudaStream_t st);
 template <typename C> void col_pass(int L, int mode, const ColPassArgs& a, cudaStream_t st);
 template <typename C>
-void conv_apply(const ConvPlan& p, int nrhs, const C* u, C* y, const double* plane_dirs, bool add_u,
-                void* scratch1, void* scratch2, cudaStream_t st);
+void conv_apply(const ConvPlan& p, int nrhs, const C* u, C* y, void* scratch1, void* scratch2, cudaStream_t st);
 // y = (I + K omega^2 m) u in float-float arithmetic with FP64 input and output; with
 // sub != null, y = sub - (I + K omega^2 m) u (the residual)
 void conv_apply_ff(const ConvPlan& p, int nrhs, const double2* u, double2* y, const double2* sub, void* scratch1,
                    void* scratch2, cudaStream_t st);
-// g = K(-omega^2 m u_inc) for plane waves (the right-hand side), float-float passes, FP64 g
-// phase: scratch of nrhs * d * n float-float complex entries (4 floats each)
-void conv_rhs_ff(const ConvPlan& p, int nrhs, const double* plane_dirs, double2* g, void* scratch1, void* scratch2,
-                 void* phase, cudaStream_t st);
+// g = K(-omega^2 m u_inc) for plane waves (the right-hand side), FP64 (f64) or float-float passes,
+// FP64 g; phase: scratch of nrhs * d * n 16-byte entries
+void conv_rhs(const ConvPlan& p, int nrhs, const double* plane_dirs, double2* g, bool f64, void* scratch1, void* scratch2,
+              void* phase, cudaStream_t st);
 // C -= A B on the complex FP32 fronts of a level on the tensor cores (tc_gemm.cu): A, B, C
 // are the blocks [r0,r1)x[k0,k1), [k0,k1)x[c0,c1), [r0,r1)x[c0,c1) of each column-major
 // front (ld = fmax, fstride elements apart); *err = 2 if a bounded wait expired
@@ -83,10 +76,12 @@ void tc_sweep_gemm(const float2* F, long fstride, int fmax, int nf, int r0, int 
 bool tc_enabled();
 // float-float copy of count FP64 reals (dst: 2 * count floats)
 void to_ff(const double* src, void* dst, long count, cudaStream_t st);
+void to_ffp(const double2* src, void* dst, long count, cudaStream_t st);  // complex tables of the passes
 size_t conv_scratch1_elems(int d, int n, int nrhs);
-// the FP32 passes' per-pass twiddle table for lines of length L (layout in fft_plan.h),
-// computed in FP64
-void fft_twiddles(int L, std::vector<double2>& tw);
+// the passes' twiddle table for lines of length L (layout in fft_lines.h; wide: 16-byte values),
+// and the symbol transforms' (layout in fft_plan.h), computed in FP64
+void line_twiddles(int L, bool wide, std::vector<double2>& tw);
+void symbol_twiddles(int L, std::vector<double2>& tw);
 size_t conv_scratch2_elems(int d, int n, int nrhs);
 void build_kernel_table(int d, int n, double omega, double h, double2* ktq, cudaStream_t st);
 // Sec. 5: g_r = q_r K delta_{p_r} / h^d for nrhs point sources (pts: nrhs x d grid indices;
@@ -98,7 +93,8 @@ void far_field(int d, int n, int nrhs, int nobs, const double2* us, const double
 size_t far_scratch_elems(int d, int n, int nrhs, int nobs);  // scratch: tables and partial sums
 void point_source(int d, int n, int nrhs, const int* pts, const double2* q, const double2* ktq, double h, double2* g,
                   cudaStream_t st);
-void build_symbol(const ConvPlan& p, const double2* ktq, double2* sym64, float2* sym32, double2* work,
+// the symbol's quadrant (fft_symbol.cu); work: (2n)^d entries, tw: symbol_twiddles(2n) on the device
+void build_symbol(int d, int n, const double2* ktq, double2* sym64, float2* sym32, double2* work, const double2* tw,
                   cudaStream_t st);
 
 // ---------------------------------------------------------------- stencils (setup.cpp)

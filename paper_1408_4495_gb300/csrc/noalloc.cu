@@ -86,8 +86,8 @@ extern "C" ls_status ls_apply_noalloc(ls_ctx* c, int nrhs, const double* x, doub
     if (s2 && ((s1 * sizeof(double2) + 255) / 256) * 256 + s2 * sizeof(double2) > kScratchBytes)
       LS_FAIL(ls::EINVAL_, "ls_apply_noalloc: scratch too small for %d right-hand sides", nrhs);
     const cudaStream_t st = ls::ctx_stream(c);
-    ls::conv_apply<double2>(*p, nrhs, reinterpret_cast<const double2*>(x), reinterpret_cast<double2*>(y), nullptr,
-                            true, t1, t2, st);
+    ls::conv_apply<double2>(*p, nrhs, reinterpret_cast<const double2*>(x), reinterpret_cast<double2*>(y), t1, t2,
+                            st);
     LS_CUDA(cudaStreamSynchronize(st));
     return LS_OK;
   } catch (const ls::Error& e) {
