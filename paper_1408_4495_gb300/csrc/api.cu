@@ -231,6 +231,45 @@ void copy_out(ls_ctx* c, void* dst, const void* src, size_t bytes, cudaStream_t 
                           st ? st : c->st));
 }
 
+// Arrays of complex doubles on the context's own device, 16-byte aligned, are read and written in
+// place by the kernels (a copy each way cost as much as a third of a large FP32 apply: 2D n = 512,
+// 16 vectors 240 -> 175 us with the casts fused as well); any other array goes through a
+// buffer of the context.
+bool in_place(const ls_ctx* c, const void* p, uintptr_t align = 16) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == c->device && reinterpret_cast<uintptr_t>(p) % align == 0;
+}
+// n doubles (directions) on the device
+const double* input_reals(ls_ctx* c, const char* name, const double* src, size_t n, cudaStream_t st, bool copy = false) {
+  if (!copy && in_place(c, src, sizeof(double))) return src;
+  double* x = buf<double>(c, name, n);
+  copy_in(c, x, src, n * sizeof(double), st);
+  return x;
+}
+bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return x < y + b_bytes && y < x + a_bytes;
+}
+// the device array with the caller's n complex numbers; copy: into the buffer in any case
+const double2* input(ls_ctx* c, const char* name, const void* src, size_t n, bool copy = false) {
+  if (!copy && in_place(c, src)) return static_cast<const double2*>(src);
+  double2* x = buf<double2>(c, name, n);
+  copy_in(c, x, src, n * sizeof(double2));
+  return x;
+}
+// the device array that a kernel writes the caller's n complex numbers to, and its copy to the
+// caller when it is not the caller's own
+double2* output(ls_ctx* c, const char* name, void* dst, size_t n) {
+  return in_place(c, dst) ? static_cast<double2*>(dst) : buf<double2>(c, name, n);
+}
+void finish(ls_ctx* c, void* dst, const double2* y, size_t n, cudaStream_t st = nullptr) {
+  if (y != dst) copy_out(c, dst, y, n * sizeof(double2), st);
+}
+
 // waits for an enqueued factorization and reads its error flag (throws on failure)
 void factor_wait(ls_ctx* c) {
   if (!c->factor_pending) return;
@@ -280,6 +319,14 @@ template <typename C> void op_apply(ls_ctx* c, int nrhs, const C* u, C* y) {
   void* t1 = buf<C>(c, sizeof(C) == 8 ? "conv1_32" : "conv1_64", s1);
   void* t2 = s2 ? buf<C>(c, sizeof(C) == 8 ? "conv2_32" : "conv2_64", s2) : nullptr;
   ls::conv_apply<C>(c->plan, nrhs, u, y, t1, t2, c->st);
+}
+
+// the FP32 operator on FP64 vectors, rounded to FP32 as they are read
+void op_apply_f32(ls_ctx* c, int nrhs, const double2* u, double2* y) {
+  const size_t s1 = ls::conv_scratch1_elems(c->d, c->n, nrhs), s2 = ls::conv_scratch2_elems(c->d, c->n, nrhs);
+  void* t1 = buf<float2>(c, "conv1_32", s1);
+  void* t2 = s2 ? buf<float2>(c, "conv2_32", s2) : nullptr;
+  ls::conv_apply_f32(c->plan, nrhs, u, y, t1, t2, c->st);
 }
 
 // y = (I + K omega^2 m) u, or y = sub - (I + K omega^2 m) u, in float-float arithmetic
@@ -930,8 +977,7 @@ ls_status ls_rhs_plane_wave(ls_ctx* c, int nrhs, const double* dirs, double* g_o
     if (c->laplace) throw Error{ls::ESTATE_, "plane waves need the Helmholtz kernel (omega > 0)"};
     if (nrhs < 1 || !dirs || !g_out) throw Error{ls::EINVAL_, "bad arguments"};
     const size_t tot = (size_t)nrhs * c->N;
-    double* dd = buf<double>(c, "dirs", (size_t)nrhs * c->d);
-    double2* gd = buf<double2>(c, "rhs_out", tot);
+    double2* gd = output(c, "rhs_out", g_out, tot);
     const size_t s1 = ls::conv_scratch1_elems(c->d, c->n, nrhs), s2 = ls::conv_scratch2_elems(c->d, c->n, nrhs);
     void* t1 = buf<double2>(c, "conv1_64", s1);
     void* t2 = s2 ? buf<double2>(c, "conv2_64", s2) : nullptr;
@@ -944,11 +990,11 @@ ls_status ls_rhs_plane_wave(ls_ctx* c, int nrhs, const double* dirs, double* g_o
       st = c->st2;
       LS_CUDA(cudaStreamWaitEvent(st, c->ev_factor, 0));
     }
-    copy_in(c, dd, dirs, (size_t)nrhs * c->d * sizeof(double), st);
+    const double* dd = input_reals(c, "dirs", dirs, (size_t)nrhs * c->d, st);
     // float-float passes on the mixed path, FP64 on the plain path
     ls::conv_rhs(c->plan, nrhs, dd, gd, c->prec != LS_PREC_MIXED, t1, t2,
                  buf<double2>(c, "rhs_phase", (size_t)nrhs * c->d * c->n), st);
-    copy_out(c, g_out, gd, tot * sizeof(double2), st);
+    finish(c, g_out, gd, tot, st);
     LS_CUDA(cudaStreamSynchronize(st));
     return LS_OK;
   } catch (const Error& e) {
@@ -969,7 +1015,7 @@ ls_status ls_rhs_point_source(ls_ctx* c, int nrhs, const int* points, const doub
     const size_t tot = (size_t)nrhs * c->N;
     int* pd = buf<int>(c, "src_points", np);
     double2* qd = strengths ? buf<double2>(c, "src_strengths", nrhs) : nullptr;
-    double2* gd = buf<double2>(c, "rhs_out", tot);
+    double2* gd = output(c, "rhs_out", g_out, tot);
     // with a factorization in flight, on the side stream (it reads only the kernel table)
     cudaStream_t st = c->st;
     if (c->factor_pending) {
@@ -979,7 +1025,7 @@ ls_status ls_rhs_point_source(ls_ctx* c, int nrhs, const int* points, const doub
     LS_CUDA(cudaMemcpyAsync(pd, ph.data(), np * sizeof(int), cudaMemcpyHostToDevice, st));
     if (qd) copy_in(c, qd, strengths, (size_t)nrhs * sizeof(double2), st);
     ls::point_source(c->d, c->n, nrhs, pd, qd, c->ktq, c->h, gd, st);
-    copy_out(c, g_out, gd, tot * sizeof(double2), st);
+    finish(c, g_out, gd, tot, st);
     LS_CUDA(cudaStreamSynchronize(st));
     return LS_OK;
   } catch (const Error& e) {
@@ -994,16 +1040,17 @@ ls_status ls_far_field(ls_ctx* c, int nrhs, const double* dirs, const double* us
     if (c->laplace) throw Error{ls::ESTATE_, "the far-field pattern needs the Helmholtz kernel (omega > 0)"};
     if (nrhs < 1 || nobs < 1 || !dirs || !us || !obs || !out) throw Error{ls::EINVAL_, "bad arguments"};
     const size_t tot = (size_t)nrhs * c->N;
-    double* dd = buf<double>(c, "ff_dirs", (size_t)nrhs * c->d);
-    double* od = buf<double>(c, "ff_obs", (size_t)nobs * c->d);
-    double2* ud = buf<double2>(c, "ff_u", tot);
-    double2* fd = buf<double2>(c, "ff_out", (size_t)nrhs * nobs);
-    copy_in(c, dd, dirs, (size_t)nrhs * c->d * sizeof(double));
-    copy_in(c, od, obs, (size_t)nobs * c->d * sizeof(double));
-    copy_in(c, ud, us, tot * sizeof(double2));
+    const size_t nout = (size_t)nrhs * nobs;
+    // inputs that the result overlaps are copied: it is written direction by direction
+    auto hit = [&](const void* p, size_t bytes) { return overlap(p, bytes, out, nout * sizeof(double2)); };
+    const size_t nd = (size_t)nrhs * c->d, no = (size_t)nobs * c->d;
+    const double2* ud = input(c, "ff_u", us, tot, hit(us, tot * sizeof(double2)));
+    const double* dd = input_reals(c, "ff_dirs", dirs, nd, c->st, hit(dirs, nd * sizeof(double)));
+    const double* od = input_reals(c, "ff_obs", obs, no, c->st, hit(obs, no * sizeof(double)));
+    double2* fd = output(c, "ff_out", out, nout);
     double2* scratch = buf<double2>(c, "ff_scratch", ls::far_scratch_elems(c->d, c->n, nrhs, nobs));
     ls::far_field(c->d, c->n, nrhs, nobs, ud, dd, od, c->w2m64, c->omega, c->h, fd, scratch, c->st);
-    copy_out(c, out, fd, (size_t)nrhs * nobs * sizeof(double2));
+    finish(c, out, fd, nout);
     LS_CUDA(cudaStreamSynchronize(c->st));
     return LS_OK;
   } catch (const Error& e) {
@@ -1098,23 +1145,15 @@ ls_status ls_apply(ls_ctx* c, int nrhs, const double* in, double* out, ls_prec p
     check_ctx(c);
     if (nrhs < 1 || !in || !out) throw Error{ls::EINVAL_, "bad arguments"};
     const size_t tot = (size_t)nrhs * c->N;
-    double2* x = buf<double2>(c, "io_in", tot);
-    double2* y = buf<double2>(c, "io_out", tot);
-    copy_in(c, x, in, tot * sizeof(double2));
-    if (prec == LS_PREC_MIXED) {
-      float2* x32 = buf<float2>(c, "io_in32", tot);
-      float2* y32 = buf<float2>(c, "io_out32", tot);
-      ls::cast<double2, float2>(x, x32, tot, c->st);
-      op_apply<float2>(c, nrhs, x32, y32);
-      ls::cast<float2, double2>(y32, y, tot, c->st);
-    } else if (prec == LS_PREC_FF) {
-      op_apply_ff(c, nrhs, x, y, nullptr);
-    } else if (prec == LS_PREC_FP64) {
-      op_apply<double2>(c, nrhs, x, y);
-    } else {
-      throw Error{ls::EINVAL_, "unknown precision"};
-    }
-    copy_out(c, out, y, tot * sizeof(double2));
+    if (prec != LS_PREC_MIXED && prec != LS_PREC_FF && prec != LS_PREC_FP64) throw Error{ls::EINVAL_, "unknown precision"};
+    // (the last pass reads each input entry right before it writes that output entry: the same
+    // array may be both, arrays that overlap otherwise may not)
+    const double2* x = input(c, "io_in", in, tot, in != out && overlap(in, tot * sizeof(double2), out, tot * sizeof(double2)));
+    double2* y = output(c, "io_out", out, tot);
+    if (prec == LS_PREC_MIXED) op_apply_f32(c, nrhs, x, y);
+    else if (prec == LS_PREC_FF) op_apply_ff(c, nrhs, x, y, nullptr);
+    else op_apply<double2>(c, nrhs, x, y);
+    finish(c, out, y, tot);
     LS_CUDA(cudaStreamSynchronize(c->st));
     return LS_OK;
   } catch (const Error& e) {
@@ -1331,9 +1370,8 @@ ls_status ls_stencil_apply(ls_ctx* c, int nrhs, const double* in, double* out, l
     check_ctx(c);
     if (nrhs < 1 || !in || !out) throw Error{ls::EINVAL_, "bad arguments"};
     const size_t tot = (size_t)nrhs * c->N;
-    double2* x = buf<double2>(c, "io_in", tot);
-    double2* y = buf<double2>(c, "io_out", tot);
-    copy_in(c, x, in, tot * sizeof(double2));
+    const double2* x = input(c, "io_in", in, tot, overlap(in, tot * sizeof(double2), out, tot * sizeof(double2)));
+    double2* y = output(c, "io_out", out, tot);
     if (prec == LS_PREC_MIXED) {
       float2* y32 = buf<float2>(c, "io_out32", tot);
       if (c->general) {
@@ -1351,7 +1389,7 @@ ls_status ls_stencil_apply(ls_ctx* c, int nrhs, const double* in, double* out, l
       if (c->general) ls::stencil_apply_pt<double2, double2>(c->d, c->n, nrhs, x, y, 1, c->N, c->apt64, c->st);
       else ls::stencil_apply<double2, double2>(c->d, c->n, nrhs, x, y, 1, c->N, c->alpha64, c->st);
     }
-    copy_out(c, out, y, tot * sizeof(double2));
+    finish(c, out, y, tot);
     LS_CUDA(cudaStreamSynchronize(c->st));
     return LS_OK;
   } catch (const Error& e) {
@@ -1367,9 +1405,8 @@ ls_status ls_precond(ls_ctx* c, int nrhs, const double* in, double* out) {
     factor_wait(c);
     if (nrhs < 1 || !in || !out) throw Error{ls::EINVAL_, "bad arguments"};
     const size_t tot = (size_t)nrhs * c->N;
-    double2* x = buf<double2>(c, "io_in", tot);
-    double2* y = buf<double2>(c, "io_out", tot);
-    copy_in(c, x, in, tot * sizeof(double2));
+    const double2* x = input(c, "io_in", in, tot, overlap(in, tot * sizeof(double2), out, tot * sizeof(double2)));
+    double2* y = output(c, "io_out", out, tot);
     if (c->prec == LS_PREC_MIXED) {
       float2* z32 = buf<float2>(c, "io_out32", tot);
       if (c->pre_refine == 1 && !c->general) {
@@ -1384,7 +1421,7 @@ ls_status ls_precond(ls_ctx* c, int nrhs, const double* in, double* out) {
     } else {
       precond_apply<double2>(c, nrhs, x, y);
     }
-    copy_out(c, out, y, tot * sizeof(double2));
+    finish(c, out, y, tot);
     LS_CUDA(cudaStreamSynchronize(c->st));
     return LS_OK;
   } catch (const Error& e) {

@@ -34,19 +34,19 @@ namespace ls {
 
 // y = (I + K omega^2 m) u  (add_u = true)  or  y = K (omega^2 m u)  (add_u = false), or, with
 // phase != null, the right-hand side g = K(-omega^2 m u_I) of the plane waves whose per-axis
-// phase tables it holds (FP64 or float-float).  C is the arithmetic of the passes; in float-float
-// the first pass reads and the last one writes FP64 (u, y, sub), and sub != null gives
-// y = sub - (...).
+// phase tables it holds (FP64 or float-float).  C is the arithmetic of the passes; in float-float,
+// and in FP32 with io64, the first pass reads and the last one writes FP64 (u, y, sub), and
+// sub != null gives y = sub - (...) (float-float).
 template <typename C>
 static void conv_run(const ConvPlan& p, int nrhs, const void* u, void* y, bool add_u, const void* sub, const void* tw,
                      const void* sym, const void* w2m, void* scratch1, void* scratch2, cudaStream_t st,
-                     const void* phase) {
+                     const void* phase, int io64 = 0) {
   const int n = p.n, L = 2 * n, d = p.d;
   const long rows = (d == 2) ? (long)n : (long)n * n;  // lines of one grid along the last axis
   C* T1 = reinterpret_cast<C*>(scratch1);
   RowPassArgs r{};
   r.in = u; r.out = T1; r.lines = (long)nrhs * rows; r.in_ls = n; r.out_ls = L;
-  r.pw = w2m; r.pw_lines = rows; r.tw = tw; r.phase = phase; r.d = d;
+  r.pw = w2m; r.pw_lines = rows; r.tw = tw; r.phase = phase; r.d = d; r.io64 = io64;
   row_pass<C>(L, -1, r, st);
   if (d == 2) {
     ColPassArgs c{};
@@ -74,7 +74,7 @@ static void conv_run(const ConvPlan& p, int nrhs, const void* u, void* y, bool a
   RowPassArgs q{};
   q.in = T1; q.out = y; q.lines = (long)nrhs * rows;
   q.in_ls = L; q.out_ls = n; q.tw = tw; q.addv = add_u ? u : nullptr; q.add_ls = n;
-  q.subv = sub;
+  q.subv = sub; q.io64 = io64;
   row_pass<C>(L, 1, q, st);
 }
 
@@ -84,6 +84,11 @@ void conv_apply(const ConvPlan& p, int nrhs, const C* u, C* y, void* scratch1, v
   conv_run<C>(p, nrhs, u, y, true, nullptr, f32 ? (const void*)p.tw32 : (const void*)p.tw64,
               f32 ? (const void*)p.sym32 : (const void*)p.sym64, f32 ? (const void*)p.w2m32 : (const void*)p.w2m64,
               scratch1, scratch2, st, nullptr);
+}
+
+void conv_apply_f32(const ConvPlan& p, int nrhs, const double2* u, double2* y, void* scratch1, void* scratch2,
+                    cudaStream_t st) {
+  conv_run<float2>(p, nrhs, u, y, true, nullptr, p.tw32, p.sym32, p.w2m32, scratch1, scratch2, st, nullptr, 1);
 }
 
 void conv_apply_ff(const ConvPlan& p, int nrhs, const double2* u, double2* y, const double2* sub, void* scratch1,

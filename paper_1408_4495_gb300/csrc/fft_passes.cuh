@@ -142,32 +142,36 @@ __global__ void __launch_bounds__(RowShape<C, L>::NT, RowShape<C, L>::MINB) k_ro
   line_fft<C, L, 1, false, true, SH::WARP, LAY>(v, reinterpret_cast<C*>(smem_raw) + li * LAY::LS,
                                                 static_cast<const C*>(a.tw), t);
   if (!valid) return;
-  // the added and subtracted entries of M butterflies are loaded together, before any store (the
+  // the added and subtracted entries of a butterfly are loaded together, before any store (the
   // output may be one of them)
   using A = typename std::conditional<OUT64, double2, C>::type;
+  constexpr bool F32 = std::is_same<C, float2>::value;
+  using B = typename std::conditional<F32, C, A>::type;  // FP32 arithmetic rounds addv as it is read
   const A* addv = static_cast<const A*>(a.addv);
   const A* subv = static_cast<const A*>(a.subv);
   A* out = static_cast<A*>(a.out) + line * a.out_ls;
 #pragma unroll
   for (int m = 0; m < E / RL; ++m) {
-    A add[RL / 2], sub[RL / 2];
+    B add[RL / 2], sub[RL / 2];
 #pragma unroll
     for (int r = 0; r < RL / 2; ++r) {
       const long i = line * a.add_ls + t + m * T + r * (L / RL);
-      add[r] = addv ? addv[i] : czero_l<A>();
-      if constexpr (OUT64) sub[r] = subv ? subv[i] : czero_l<A>();
+      add[r] = czero_l<B>();
+      if (addv) {
+        if constexpr (OUT64 && F32) add[r] = l_of_f64<B>(addv[i]);
+        else add[r] = addv[i];
+      }
+      if constexpr (OUT64 && !F32) sub[r] = subv ? subv[i] : czero_l<B>();
     }
 #pragma unroll
     for (int r = 0; r < RL / 2; ++r) {
-      C x = v[m * RL + r];
+      const C x = v[m * RL + r];
       A o;
-      if constexpr (OUT64) {
-        if constexpr (std::is_same<C, float2>::value) {
-          x = l_add(x, l_of_f64<C>(add[r]));
-          o = make_double2(f64_of(x.x), f64_of(x.y));
-        } else {
-          o = l_add(l_to_f64(x), add[r]);
-        }
+      if constexpr (OUT64 && F32) {
+        const C y = l_add(x, add[r]);
+        o = make_double2(f64_of(y.x), f64_of(y.y));
+      } else if constexpr (OUT64) {
+        o = l_add(l_to_f64(x), add[r]);
         if (subv) o = l_sub(sub[r], o);
       } else {
         o = l_norm(l_add(x, add[r]));
@@ -297,9 +301,13 @@ template <typename C, int L> void launch_row_L(int sign, const RowPassArgs& a, c
       else LS_FAIL(EINVAL_, "row pass: no plane waves in FP32");
     } else if constexpr (FF) {
       launch_row_fwd<C, L, ROW_IN_F64>(a, st);
+    } else if (F32 && a.io64) {
+      if constexpr (F32) launch_row_fwd<C, L, ROW_IN_F64>(a, st);
     } else {
       launch_row_fwd<C, L, ROW_IN_C>(a, st);
     }
+  } else if (F32 && a.io64) {
+    if constexpr (F32) launch_row_inv<C, L, true>(a, st);
   } else {
     launch_row_inv<C, L, FF>(a, st);
   }

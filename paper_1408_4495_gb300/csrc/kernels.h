@@ -23,6 +23,7 @@ struct RowPassArgs {
   const void* addv;    // inverse: out += addv[line * add_ls + e], or null
   long add_ls;
   const void* subv;    // inverse: out = subv - (...), or null (FP64 output only)
+  int io64;            // FP32 passes: in (forward) / addv and out (inverse) are FP64
 };
 
 struct ColPassArgs {
@@ -53,6 +54,9 @@ template <typename C> void row_pass(int L, int sign, const RowPassArgs& a, cudaS
 template <typename C> void col_pass(int L, int mode, const ColPassArgs& a, cudaStream_t st);
 template <typename C>
 void conv_apply(const ConvPlan& p, int nrhs, const C* u, C* y, void* scratch1, void* scratch2, cudaStream_t st);
+// the FP32 passes with FP64 u and y: u is rounded to FP32 as it is read
+void conv_apply_f32(const ConvPlan& p, int nrhs, const double2* u, double2* y, void* scratch1, void* scratch2,
+                    cudaStream_t st);
 // y = (I + K omega^2 m) u in float-float arithmetic with FP64 input and output; with
 // sub != null, y = sub - (I + K omega^2 m) u (the residual)
 void conv_apply_ff(const ConvPlan& p, int nrhs, const double2* u, double2* y, const double2* sub, void* scratch1,
