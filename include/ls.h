@@ -407,16 +407,16 @@ ls_status ls_profile_stop(char* report, int capacity);
  * how many CTAs per SM the split of a solve sweep level aims at, and the smallest FP32
  * forward and backward solve levels (rows of their products, at least 32) run on the tensor
  * cores, and the largest bottom solve level (columns of its product, up to 256; rows up to
- * 64) run one CTA per front.  The last three default to -1, automatic per solve: tensor-core
- * levels from 64 rows in 3D or with more than 16 right-hand sides, none for at most 16 in
- * 2D; one-CTA-per-front levels up to 256 columns with more than 16 right-hand sides, up to
- * 64 with at most 16.  A coordinate search
+ * 64) run one CTA per front.  The last three default to -1, automatic by the level's size:
+ * tensor-core levels from 64 rows where the level's product has at least 2^25 complex terms;
+ * one-CTA-per-front levels up to 64 columns, up to 256 on levels of 512 fronts and more with
+ * more than 16 right-hand sides.  A coordinate search
  * keeps each alternative that is more than 2 % faster (the fastest of 2 factorizations / 3
  * solves of nrhs right-hand sides, CUDA events).  The choice is applied to c, kept for every
  * later context of the same (dim, n, prec, kernel) in this process, and, when the
  * environment variable LS_TUNE_FILE names a file, written there (one JSON object per line)
  * and read back by the first ls_setup of a later process.  Leaves c factored (with the
- * chosen shapes).  FFT radices (8, 4, 2, 3) and the right-hand-side batch widths (16 per
+ * chosen shapes).  FFT factors and the right-hand-side batch widths (16 per
  * item, 64 per launch) are fixed.
  *   nrhs     right-hand sides of the timed solves, >= 1.
  *   report   NUL-terminated JSON: the choice and every timing (truncated to capacity bytes;

@@ -42,6 +42,7 @@
 #include <map>
 #include <memory>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "alloc.h"
@@ -727,19 +728,65 @@ __global__ void __launch_bounds__(512) k_panel(LevelK<C> L, int k0, int k1, int*
   }
 }
 
+// Runs body(W, i) for i = 0 .. w - 1 (w <= NB) in four loops of eight with W = NB, NB - 8, ..: the
+// values of W columns (or rows) live in registers, the current one first, and every step moves
+// them down by one as it updates them.  A fully unrolled triangle does less arithmetic, but its
+// straight-line code (40 KB and more, run once per launch) waits for instruction fetches most of
+// the time: TRSMTIMES
+template <int W, typename F> __device__ __forceinline__ void rolling_steps(int i0, int w, F&& body) {
+  const int i1 = min(w, i0 + 8);
+#pragma unroll 1
+  for (int i = i0; i < i1; ++i) body(std::integral_constant<int, W>{}, i);
+  if constexpr (W > 8) rolling_steps<W - 8>(i0 + 8, w, body);
+}
+
+// Triangle staged for solve_rolling: T[i * NB + j], j > i, the factor of x_i in the update of x_j;
+// src(i, j) its global address.  Entries past the triangle only enter values that are not used.
+constexpr int TRI_SIZE = NB * NB + NB;
+template <typename C, typename F> __device__ __forceinline__ void load_triangle(C* T, int w, F src) {
+  constexpr int B = 8;  // loads in flight per thread
+  for (int base = threadIdx.x; base < w * w; base += blockDim.x * B) {
+    C v[B];
+#pragma unroll
+    for (int u = 0; u < B; ++u) {
+      const int e = base + u * blockDim.x;
+      if (e < w * w) v[u] = *src(e / w, e % w);
+    }
+#pragma unroll
+    for (int u = 0; u < B; ++u) {
+      const int e = base + u * blockDim.x;
+      if (e < w * w) T[(e / w) * NB + e % w] = v[u];
+    }
+  }
+}
+
+// x_i final (times rd_i with DIAG), then x_j -= T_ij x_i for j > i (right-looking: one dependent
+// product per step); store(i, x_i)
+template <bool DIAG, typename C, typename F>
+__device__ __forceinline__ void solve_rolling(C* x, const C* T, const C* rd, int w, F store) {
+  rolling_steps<NB>(0, w, [&](auto width, int i) {
+    constexpr int W = decltype(width)::value;
+    const C* t = T + i * NB + i;
+    const C xi = DIAG ? cmul(x[0], rd[i]) : x[0];
+    store(i, xi);
+#pragma unroll
+    for (int r = 1; r < W; ++r) x[r - 1] = cfms(x[r], t[r], xi);
+  });
+}
+
+constexpr int TRSM_COLS = 64;  // columns (or ring rows) per CTA: a front with few spreads over more SMs
+
 // Columns c in [k1, ncols): apply the panel's row swaps, then F[k0:k1, c] = L_kk^{-1} F[k0:k1, c].
-template <typename C> __global__ void __launch_bounds__(128) k_trsm_lower(LevelK<C> L, int k0, int k1) {
+template <typename C> __global__ void __launch_bounds__(TRSM_COLS) k_trsm_lower(LevelK<C> L, int k0, int k1) {
   const int z = blockIdx.x;
   const int fmax = L.fmax, w = k1 - k0;
   C* A = L.F + (size_t)z * fmax * L.ncols;
-  __shared__ C Ld[NB][NB + 1];
+  __shared__ C T[TRI_SIZE];
   // net effect of the panel's row swaps: position pos[i] receives original row src[i];
   // positions k0..k1-1 first, then the pivot rows below k1 that were swapped up
   __shared__ int pos[2 * NB], src[2 * NB], npos, pv[NB];
-  for (int idx = threadIdx.x; idx < w * w; idx += blockDim.x) {
-    const int i = idx % w, l = idx / w;
-    Ld[i][l] = A[(size_t)(k0 + l) * fmax + k0 + i];
-  }
+  const C* P = A + (size_t)k0 * fmax + k0;
+  load_triangle<C>(T, w, [&](int i, int j) { return P + (size_t)i * fmax + j; });
   for (int j = threadIdx.x; j < w; j += blockDim.x) pv[j] = L.piv[(size_t)z * L.smax + k0 + j];
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -765,8 +812,7 @@ template <typename C> __global__ void __launch_bounds__(128) k_trsm_lower(LevelK
   const int np = npos;
   C x[NB];
 #pragma unroll
-  for (int i = 0; i < NB; ++i)
-    if (i < w) x[i] = col[src[i]];
+  for (int i = 0; i < NB; ++i) x[i] = i < w ? col[src[i]] : czero<C>();
   {
     C extra[NB];
 #pragma unroll
@@ -776,61 +822,34 @@ template <typename C> __global__ void __launch_bounds__(128) k_trsm_lower(LevelK
     for (int i = 0; i < NB; ++i)
       if (w + i < np) col[pos[w + i]] = extra[i];
   }
-  // column-oriented (right-looking): x_i final, then every x_r below it updated at once
-#pragma unroll
-  for (int i = 0; i < NB - 1; ++i) {
-    if (i < w) {
-#pragma unroll
-      for (int r = i + 1; r < NB; ++r)
-        if (r < w) x[r] = cfms(x[r], Ld[r][i], x[i]);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < NB; ++i)
-    if (i < w) col[k0 + i] = x[i];
+  solve_rolling<false>(x, T, (const C*)nullptr, w, [&](int i, C v) { col[k0 + i] = v; });
 }
 
-// Columns c in [smax, ncols): F[j0:j1, c] = U_blk^{-1} F[j0:j1, c] (non-unit upper).
-// Column-oriented (right-looking) substitution: once x_i is final, every x_l above it takes
-// its update at once, so a thread's dependent chain is one product per row (the dot-product
-// form chains up to 31 products per row); the reciprocals of the diagonal are formed once
-// per CTA.
-template <typename C> __global__ void __launch_bounds__(128) k_trsm_upper(LevelK<C> L, int j0, int j1) {
+// Columns c in [smax, ncols): F[j0:j1, c] = U_blk^{-1} F[j0:j1, c] (non-unit upper), from the last
+// row up; the reciprocals of the diagonal are formed once per CTA.
+template <typename C> __global__ void __launch_bounds__(TRSM_COLS) k_trsm_upper(LevelK<C> L, int j0, int j1) {
   const int z = blockIdx.x;
   const int fmax = L.fmax, w = j1 - j0;
   C* A = L.F + (size_t)z * fmax * L.ncols;
-  __shared__ C Ud[NB][NB + 1];
+  __shared__ C T[TRI_SIZE];
   __shared__ C rdg[NB];
-  for (int idx = threadIdx.x; idx < w * w; idx += blockDim.x) {
-    const int i = idx % w, l = idx / w;
-    Ud[i][l] = A[(size_t)(j0 + l) * fmax + j0 + i];
-  }
+  const C* U = A + (size_t)(j1 - 1) * fmax + j1 - 1;  // the last diagonal entry
+  load_triangle<C>(T, w, [&](int i, int j) { return U - (size_t)i * fmax - j; });
   __syncthreads();
   if (threadIdx.x < w) {
     C one;
     one.x = 1;
     one.y = 0;
-    rdg[threadIdx.x] = cdiv(one, Ud[threadIdx.x][threadIdx.x]);
+    rdg[threadIdx.x] = cdiv(one, T[threadIdx.x * NB + threadIdx.x]);
   }
   __syncthreads();
   const int c = L.smax + blockIdx.y * blockDim.x + threadIdx.x;
   if (c >= L.ncols) return;
-  C* col = A + (size_t)c * fmax;
+  C* col = A + (size_t)c * fmax + j1 - 1;
   C x[NB];
 #pragma unroll
-  for (int i = 0; i < NB; ++i)
-    if (i < w) x[i] = col[j0 + i];
-#pragma unroll
-  for (int i = NB - 1; i >= 0; --i) {
-    if (i < w) {
-      x[i] = cmul(x[i], rdg[i]);
-#pragma unroll
-      for (int l = 0; l < i; ++l) x[l] = cfms(x[l], Ud[l][i], x[i]);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < NB; ++i)
-    if (i < w) col[j0 + i] = x[i];
+  for (int i = 0; i < NB; ++i) x[i] = i < w ? col[-i] : czero<C>();
+  solve_rolling<true>(x, T, rdg, w, [&](int i, C v) { col[-i] = v; });
 }
 
 // Ring rows r in [smax, fmax) of every front, panel columns [k0, k1): the multipliers
@@ -841,19 +860,17 @@ template <typename C> __global__ void __launch_bounds__(128) k_trsm_upper(LevelK
 // Y = -L21 L11^{-1} P are formed backward stably (the product F21 [H | F11^{-1}] of the
 // explicit inverse would amplify rounding by cond(F11)).  One thread per ring row; U_kk and
 // its reciprocal pivots in shared memory.
-template <typename C> __global__ void __launch_bounds__(256) k_ring_trsm(LevelK<C> L, int k0, int k1) {
+template <typename C> __global__ void __launch_bounds__(TRSM_COLS) k_ring_trsm(LevelK<C> L, int k0, int k1) {
   using Rl = typename RealOf<C>::T;
-  __shared__ C u[NB][NB + 1];  // u[j][i] = U_kk(i, j)
+  __shared__ C T[TRI_SIZE];
   __shared__ C invd[NB];
   const int z = blockIdx.x, w = k1 - k0, fmax = L.fmax;
   C* A = L.F + (size_t)z * fmax * L.ncols;
-  for (int e = threadIdx.x; e < w * w; e += blockDim.x) {
-    const int i = e % w, j = e / w;
-    u[j][i] = A[(size_t)(k0 + j) * fmax + k0 + i];
-  }
+  const C* U = A + (size_t)k0 * fmax + k0;
+  load_triangle<C>(T, w, [&](int i, int j) { return U + (size_t)j * fmax + i; });
   __syncthreads();
   for (int j = threadIdx.x; j < w; j += blockDim.x) {
-    const C dg = u[j][j];
+    const C dg = T[j * NB + j];
     const Rl den = cabs2(dg);
     C inv;
     inv.x = den > 0 ? dg.x / den : (Rl)0;
@@ -867,25 +884,13 @@ template <typename C> __global__ void __launch_bounds__(256) k_ring_trsm(LevelK<
   C f[NB];
 #pragma unroll
   for (int c = 0; c < NB; ++c) f[c] = c < w ? row[(size_t)c * fmax] : czero<C>();
-  // column-oriented (right-looking): f_c final, then every f_c2 right of it updated at once
-#pragma unroll
-  for (int c = 0; c < NB; ++c) {
-    if (c < w) {
-      f[c] = cmul(f[c], invd[c]);
-#pragma unroll
-      for (int c2 = c + 1; c2 < NB; ++c2)
-        if (c2 < w) f[c2] = cfms(f[c2], f[c], u[c2][c]);
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < NB; ++c)
-    if (c < w) row[(size_t)c * fmax] = f[c];
+  solve_rolling<true>(f, T, invd, w, [&](int i, C v) { row[(size_t)i * fmax] = v; });
 }
 
 template <typename C> static void launch_ring_trsm(const LevelK<C>& L, int k0, int k1, cudaStream_t st) {
   if (L.bmax <= 0) return;
   LS_LAUNCH(sizeof(C) == 8 ? "nd_trsm_c64" : "nd_trsm_c128", st,
-            k_ring_trsm<C><<<dim3(L.nf, (L.bmax + 255) / 256), 256, 0, st>>>(L, k0, k1));
+            k_ring_trsm<C><<<dim3(L.nf, (L.bmax + TRSM_COLS - 1) / TRSM_COLS), TRSM_COLS, 0, st>>>(L, k0, k1));
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1037,6 +1042,165 @@ __global__ void __launch_bounds__(panel_reg_rows<C>()) k_panel_reg(LevelK<C> L, 
   if (r == 0) swp[(size_t)z * SWP_STRIDE] = min(cnt, 2 * NB);
 }
 
+// reciprocal of a pivot entry (0 for a zero pivot)
+template <typename C> __device__ __forceinline__ C pivot_inverse(C a) {
+  using Rl = typename RealOf<C>::T;
+  const Rl den = cabs2(a), rden = den > 0 ? recip(den) : (Rl)0;
+  C inv;
+  inv.x = a.x * rden;
+  inv.y = -a.y * rden;
+  return inv;
+}
+
+// The panel of fronts with at most 128 own rows: four neighbouring threads share a row, thread g with
+// the columns c = g (mod 4) in registers, the current block of four columns first.  A column takes
+// two barriers: after the first every thread knows the pivot row from the warps' keys, and its
+// threads write the row (with the pivot's reciprocal) to shared memory; after the second the
+// column's owner passes the row's multiplier to the other threads of the row, which update their
+// columns, the next one first, whose key is reduced while the others are updated.  Bound by the
+// latency of that chain, which a fourth of the instructions per thread shortens: 64 rows 22.4 -> 15
+// us a panel (larger fronts gain nothing: their warps fill the issue slots either way).  Keys,
+// positions and swp as in k_panel_reg; the rows of U go to their positions as they are chosen, the
+// multipliers wait in shared memory until the positions of all rows are known.
+// Runs body(W, b) for the blocks b = 0 .. nb - 1 of G columns, W the local columns still live (in
+// quarters of NC: code for every width would be fetched more slowly than the work it saves)
+template <int NC, int W, typename F> __device__ __forceinline__ void panel_blocks(int b0, int nb, F&& body) {
+  constexpr int Q = NC / 4;
+  const int b1 = min(nb, b0 + Q);
+#pragma unroll 1
+  for (int b = b0; b < b1; ++b) body(std::integral_constant<int, W>{}, b);
+  if constexpr (W > Q) panel_blocks<NC, W - Q>(b0 + Q, nb, body);
+}
+
+// The columns of one row held by thread g of its G threads, and the update by pivot row prow
+// (entries from the block's first column on) with the row's multiplier m for column g0 of the
+// block; the last column of a block moves the registers down.  next(x) is called with this
+// thread's entry of the following column as soon as it is known.
+template <int G, int W, int g0, typename C, typename N>
+__device__ __forceinline__ void panel_update(C* a, C m, const C* prow, int g, N next) {
+  if constexpr (g0 < G - 1) {
+    const C u = cfms(a[0], m, prow[g]);
+    if (g > g0) a[0] = u;
+    next(a[0]);
+#pragma unroll
+    for (int l = 1; l < W; ++l) a[l] = cfms(a[l], m, prow[l * G + g]);
+  } else {
+    if constexpr (W > 1) a[0] = cfms(a[1], m, prow[G + g]);
+    next(a[0]);
+#pragma unroll
+    for (int l = 2; l < W; ++l) a[l - 1] = cfms(a[l], m, prow[l * G + g]);
+  }
+}
+template <int g, int G, typename F> __device__ __forceinline__ void panel_cols(F&& f) {
+  f(std::integral_constant<int, g>{});
+  if constexpr (g + 1 < G) panel_cols<g + 1, G>(f);
+}
+
+constexpr int PS_ROWS = 128;  // at most
+template <typename C>
+__global__ void __launch_bounds__(4 * PS_ROWS) k_panel_small(LevelK<C> L, int k0, int k1, int* __restrict__ swp, int* err) {
+  constexpr int G = 4;
+  constexpr int NC = NB / G, RPW = 32 / G;  // columns per thread, rows per warp
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* Ls = reinterpret_cast<C*>(smem_raw);  // [w][rows of the CTA] multipliers
+  __shared__ __align__(16) C prow[NB];  // the pivot row from the current block on, with the pivot's reciprocal
+  __shared__ C pdiag;                      // and the pivot
+  __shared__ unsigned skey[2][32];
+  __shared__ int jps[PS_ROWS], posn[PS_ROWS];  // per row: the column it was chosen at (-1: none), its final position
+  __shared__ int vac[NB];
+  __shared__ int wcnt[32];
+  __shared__ int cnt;
+  const int z = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+  const int r = tid / G, g = tid % G, rows = nw * RPW;
+  const int fmax = L.fmax, R = L.smax - k0, w = k1 - k0;
+  C* A = L.F + (size_t)z * fmax * L.ncols + (size_t)k0 * fmax + k0;  // local (r, c) at A[c * fmax + r]
+  C a[NC];
+#pragma unroll
+  for (int l = 0; l < NC; ++l) {
+    const int c = g + l * G;
+    a[l] = (r < R && c < w) ? A[(size_t)c * fmax + r] : czero<C>();
+  }
+  if (tid == 0) cnt = 0;
+  if (tid < NB) vac[tid] = tid;
+  if (g == 0) jps[r] = -1;
+  bool live = r < R;
+  auto publish_key = [&](C x, int gn, int par) {
+    const unsigned mag = __float_as_uint((float)(fabs(x.x) + fabs(x.y)));
+    const unsigned kw =
+        __reduce_max_sync(0xffffffffu, live && g == gn ? ((mag >> 9) << 10) | (1023u - (unsigned)r) : 0u);
+    if (lane == 0) skey[par][wid] = kw;
+  };
+  publish_key(a[0], 0, 0);
+  panel_blocks<NC, NC>(0, (w + G - 1) / G, [&](auto width, int b) {
+    constexpr int W = decltype(width)::value;
+    panel_cols<0, G>([&](auto col) {
+      constexpr int g0 = decltype(col)::value;
+      const int j = b * G + g0, par = j & 1;
+      if (j >= w) return;
+      __syncthreads();  // the keys of column j; the updates of column j - 1 have read prow
+      const unsigned km = __reduce_max_sync(0xffffffffu, lane < nw ? skey[par][lane] : 0u);
+      if ((km >> 10) == 0u && tid == 0) atomicCAS(err, 0, 1);  // zero pivot, or no live row left
+      const int bi = km != 0u ? 1023 - (int)(km & 1023u) : -1;
+      if (r == bi) {
+        live = false;
+        if (g == g0) {
+          jps[r] = j;
+          pdiag = a[0];
+        }
+        const C first = g == g0 ? pivot_inverse(a[0]) : a[0];
+        prow[g] = first;
+#pragma unroll
+        for (int l = 1; l < W; ++l) prow[l * G + g] = a[l];
+      }
+      __syncthreads();
+      const bool on = live && bi >= 0;
+      C m = on ? cmul(a[0], prow[g0]) : czero<C>();
+      m = shfl_c(m, (lane & ~(G - 1)) | g0);
+      if (live && g == g0) Ls[j * rows + r] = on ? m : a[0];
+      panel_update<G, W, g0>(a, m, prow, g, [&](C x) { publish_key(x, (g0 + 1) % G, par ^ 1); });
+      // the row of U
+      if (wid == j % nw && bi >= 0 && lane < w - j) A[(size_t)(j + lane) * fmax + j] = lane == 0 ? pdiag : prow[g0 + lane];
+    });
+  });
+  __syncthreads();  // jps
+  // one thread per row: positions >= w vacated by pivots, in increasing order
+  const int row = tid;
+  const bool has = row < R;
+  const int jp = has ? jps[row] : -1;
+  const bool vp = jp >= 0 && row >= w;
+  const unsigned bv = __ballot_sync(0xffffffffu, vp);
+  if (lane == 0) wcnt[wid] = __popc(bv);
+  __syncthreads();
+  const unsigned lt = (1u << lane) - 1u;
+  if (vp) {
+    int before = 0;
+    for (int q = 0; q < wid; ++q) before += wcnt[q];
+    vac[before + __popc(bv & lt)] = row;
+  }
+  __syncthreads();
+  // rows at positions < w not chosen (all in warp 0) take the vacated positions in order
+  const bool dp = has && jp < 0 && row < w;
+  const unsigned bd = __ballot_sync(0xffffffffu, dp);
+  const int pos = jp >= 0 ? jp : (dp ? min(vac[__popc(bd & lt)], R - 1) : row);
+  if (has) {
+    posn[row] = pos;
+    if (pos != row) {
+      const int q = atomicAdd(&cnt, 1);
+      if (q < 2 * NB) {
+        swp[(size_t)z * SWP_STRIDE + 1 + 2 * q] = pos;
+        swp[(size_t)z * SWP_STRIDE + 2 + 2 * q] = row;
+      }
+    }
+  }
+  __syncthreads();
+  if (tid == 0) swp[(size_t)z * SWP_STRIDE] = min(cnt, 2 * NB);
+  // the multipliers (a chosen row has them up to its column); consecutive threads, consecutive rows
+  for (int e = tid; e < w * rows; e += blockDim.x) {
+    const int c = e / rows, i = e - c * rows;
+    if (i < R && (jps[i] < 0 || c < jps[i])) A[(size_t)c * fmax + posn[i]] = Ls[e];
+  }
+}
+
 // Panel [k0, k1) of a front with up to PC_CTAS * 512 own rows (FP32): the register panel
 // spread over a thread-block cluster, one own row per thread, 512 rows per CTA.  Per column:
 // each warp's best live row publishes its key, reciprocal pivot and row to its CTA's
@@ -1174,44 +1338,41 @@ __global__ void __launch_bounds__(PC_ROWS) k_panel_cluster(LevelK<C> L, int k0, 
 // Columns c in [c0, c1): apply the panel's row permutation given as (position, source)
 // pairs local to k0 (k_panel_reg / k_panel_cluster; none when swp is null), then
 // F[k0:k1, c] = L_kk^{-1} F[k0:k1, c].
-template <typename C> __global__ void __launch_bounds__(128) k_trsm_lower_swp(LevelK<C> L, int k0, int k1, int c0,
-                                                                              int c1, const int* __restrict__ swp) {
+template <typename C> __global__ void __launch_bounds__(TRSM_COLS) k_trsm_lower_swp(LevelK<C> L, int k0, int k1, int c0,
+                                                                                    int c1, const int* __restrict__ swp) {
   const int z = blockIdx.x;
   const int fmax = L.fmax, w = k1 - k0, R = L.smax - k0;
   C* A = L.F + (size_t)z * fmax * L.ncols;
-  __shared__ C Ld[NB][NB + 1];
+  __shared__ C T[TRI_SIZE];
   __shared__ int stop[NB], bpos[NB], bsrc[NB], nb;
-  for (int idx = threadIdx.x; idx < w * w; idx += blockDim.x) {
-    const int i = idx % w, l = idx / w;
-    Ld[i][l] = A[(size_t)(k0 + l) * fmax + k0 + i];
-  }
+  const int* sw = swp ? swp + (size_t)z * SWP_STRIDE : nullptr;
+  const int cnt = sw ? min(sw[0], 2 * NB) : 0;
+  const C* P = A + (size_t)k0 * fmax + k0;
+  load_triangle<C>(T, w, [&](int i, int j) { return P + (size_t)i * fmax + j; });
   if (threadIdx.x < NB) stop[threadIdx.x] = threadIdx.x;
+  if (threadIdx.x == 0) nb = 0;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const int* sw = swp ? swp + (size_t)z * SWP_STRIDE : nullptr;
-    const int cnt = sw ? min(sw[0], 2 * NB) : 0;
-    int m = 0;
-    for (int qq = 0; qq < cnt; ++qq) {
-      const int ps = sw[1 + 2 * qq], sr = sw[2 + 2 * qq];
-      if (ps < 0 || ps >= R || sr < 0 || sr >= R) continue;
-      if (ps < w) stop[ps] = sr;
-      else if (m < NB) {
+  for (int q = threadIdx.x; q < cnt; q += blockDim.x) {
+    const int ps = sw[1 + 2 * q], sr = sw[2 + 2 * q];
+    if (ps < 0 || ps >= R || sr < 0 || sr >= R) continue;
+    if (ps < w) {
+      stop[ps] = sr;
+    } else {
+      const int m = atomicAdd(&nb, 1);  // (the moves below the panel are independent: any order)
+      if (m < NB) {
         bpos[m] = ps;
         bsrc[m] = sr;
-        ++m;
       }
     }
-    nb = m;
   }
   __syncthreads();
   const int c = c0 + blockIdx.y * blockDim.x + threadIdx.x;
   if (c >= c1) return;
   C* col = A + (size_t)c * fmax + k0;
-  const int np = nb;
+  const int np = min(nb, NB);
   C x[NB];
 #pragma unroll
-  for (int i = 0; i < NB; ++i)
-    if (i < w) x[i] = col[stop[i]];
+  for (int i = 0; i < NB; ++i) x[i] = i < w ? col[stop[i]] : czero<C>();
   {
     C extra[NB];
 #pragma unroll
@@ -1221,18 +1382,7 @@ template <typename C> __global__ void __launch_bounds__(128) k_trsm_lower_swp(Le
     for (int i = 0; i < NB; ++i)
       if (i < np) col[bpos[i]] = extra[i];
   }
-  // column-oriented (right-looking): x_i final, then every x_r below it updated at once
-#pragma unroll
-  for (int i = 0; i < NB - 1; ++i) {
-    if (i < w) {
-#pragma unroll
-      for (int r = i + 1; r < NB; ++r)
-        if (r < w) x[r] = cfms(x[r], Ld[r][i], x[i]);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < NB; ++i)
-    if (i < w) col[i] = x[i];
+  solve_rolling<false>(x, T, (const C*)nullptr, w, [&](int i, C v) { col[i] = v; });
 }
 
 // Row permutations of nrec panels applied in order to the columns [c0, c1) (no solve): record
@@ -1677,6 +1827,25 @@ static int gj_threads(int s, int nc) {
   return std::max((s + 31) / 32 * 32, std::min(256, std::max(32, t)));
 }
 
+// the register panel: four threads per row up to PS_ROWS rows, one above
+template <typename C>
+static void launch_panel_reg(const LevelK<C>& L, int k0, int k1, int* swp, int* err, cudaStream_t st) {
+  const int R = L.smax - k0;
+  const char* cls = sizeof(C) == 8 ? "nd_panel_c64" : "nd_panel_c128";
+  if (R > PS_ROWS) {
+    LS_LAUNCH(cls, st, k_panel_reg<C><<<L.nf, (R + 31) / 32 * 32, 0, st>>>(L, k0, k1, swp, err));
+    return;
+  }
+  const int rows = (R + 7) / 8 * 8;
+  static std::atomic<bool> attr{false};  // set once per process; repeats are harmless
+  if (!attr.load(std::memory_order_acquire)) {
+    LS_CUDA(cudaFuncSetAttribute(k_panel_small<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(NB * PS_ROWS * sizeof(C))));
+    attr.store(true, std::memory_order_release);
+  }
+  LS_LAUNCH(cls, st, k_panel_small<C><<<L.nf, rows * 4, (size_t)(k1 - k0) * rows * sizeof(C), st>>>(L, k0, k1, swp, err));
+}
+
 // shared memory of the Gauss-Jordan CTA: own-row block, normalised pivot row, row order
 template <typename C> static size_t gj_smem(int s, int nc) {
   return ((size_t)s * nc + nc) * sizeof(C) + 2 * (size_t)s * sizeof(int);
@@ -1728,7 +1897,7 @@ static void reg_sweeps(const LevelK<C>& L, int* swp, int* err, const NdTune* tc,
   for (int k0 = 0; k0 < L.smax; k0 += NB) {
     const int k1 = std::min(k0 + NB, L.smax), R = L.smax - k0;
     const int r32 = (R + 31) / 32 * 32;
-    LS_LAUNCH(f32 ? "nd_panel_c64" : "nd_panel_c128", st, k_panel_reg<C><<<L.nf, r32, 0, st>>>(L, k0, k1, swp, err));
+    launch_panel_reg<C>(L, k0, k1, swp, err, st);
     launch_ring_trsm<C>(L, k0, k1, st);
     const int m = L.ncols - k1;
     const size_t smem = (size_t)(k1 - k0) * r32 * sizeof(C) + (size_t)R * sizeof(int);
@@ -1869,7 +2038,7 @@ void nd_factor_launch(NdPlan* p, const void* alpha64, const void* cint64, const 
                         k_panel<C, false><<<L.nf, 512, 0, st>>>(L, k0, k1, p->d_err));
             launch_ring_trsm<C>(L, k0, k1, st);
             LS_LAUNCH(f32 ? "nd_trsm_c64" : "nd_trsm_c128", st,
-                      k_trsm_lower<C><<<dim3(L.nf, (m + 127) / 128), 128, 0, st>>>(L, k0, k1));
+                      k_trsm_lower<C><<<dim3(L.nf, (m + TRSM_COLS - 1) / TRSM_COLS), TRSM_COLS, 0, st>>>(L, k0, k1));
             launch_gemm<C>(L, k1, L.smax, k1, L.ncols, k0, k1, st, p->d_err, tcp);
             launch_gemm<C>(L, L.smax, L.fmax, k1, L.smax, k0, k1, st, p->d_err, tcp);
           }
@@ -1883,8 +2052,7 @@ void nd_factor_launch(NdPlan* p, const void* alpha64, const void* cint64, const 
           const int k1 = std::min(k0 + NB, K1), R = L.smax - k0;
           int* rec = p->swp + (two ? np : 0) * rs;
           if (R <= panel_reg_rows<C>()) {
-            LS_LAUNCH(f32 ? "nd_panel_c64" : "nd_panel_c128", st,
-                      k_panel_reg<C><<<L.nf, (R + 31) / 32 * 32, 0, st>>>(L, k0, k1, rec, p->d_err));
+            launch_panel_reg<C>(L, k0, k1, rec, p->d_err, st);
           } else if constexpr (sizeof(C) == 8) {
             const int ncta = (R + PC_ROWS - 1) / PC_ROWS;
             cudaLaunchConfig_t cfg = {};
@@ -1905,7 +2073,7 @@ void nd_factor_launch(NdPlan* p, const void* alpha64, const void* cint64, const 
             // one level: permutation and forward substitution of every trailing column, then
             // the trailing GEMM with K = NB
             LS_LAUNCH(f32 ? "nd_trsm_c64" : "nd_trsm_c128", st,
-                      k_trsm_lower_swp<C><<<dim3(L.nf, (L.ncols - k1 + 127) / 128), 128, 0, st>>>(L, k0, k1, k1,
+                      k_trsm_lower_swp<C><<<dim3(L.nf, (L.ncols - k1 + TRSM_COLS - 1) / TRSM_COLS), TRSM_COLS, 0, st>>>(L, k0, k1, k1,
                                                                                                  L.ncols, rec));
             launch_gemm<C>(L, k1, L.smax, k1, L.ncols, k0, k1, st, p->d_err, tcp);
             launch_gemm<C>(L, L.smax, L.fmax, k1, L.smax, k0, k1, st, p->d_err, tcp);
@@ -1919,7 +2087,7 @@ void nd_factor_launch(NdPlan* p, const void* alpha64, const void* cint64, const 
           // the rest of the block: permutation, forward substitution, update below
           if (k1 < K1) {
             LS_LAUNCH(f32 ? "nd_trsm_c64" : "nd_trsm_c128", st,
-                      k_trsm_lower_swp<C><<<dim3(L.nf, (K1 - k1 + 127) / 128), 128, 0, st>>>(L, k0, k1, k1, K1, rec));
+                      k_trsm_lower_swp<C><<<dim3(L.nf, (K1 - k1 + TRSM_COLS - 1) / TRSM_COLS), TRSM_COLS, 0, st>>>(L, k0, k1, k1, K1, rec));
             launch_gemm<C>(L, k1, L.fmax, k1, K1, k0, k1, st, p->d_err, tcp);
           }
         }
@@ -1931,7 +2099,7 @@ void nd_factor_launch(NdPlan* p, const void* alpha64, const void* cint64, const 
           for (int q = 0; q < np; ++q) {
             const int k0 = K0 + q * NB, k1 = std::min(k0 + NB, K1);
             LS_LAUNCH(f32 ? "nd_trsm_c64" : "nd_trsm_c128", st,
-                      k_trsm_lower_swp<C><<<dim3(L.nf, (m + 127) / 128), 128, 0, st>>>(L, k0, k1, K1, L.ncols,
+                      k_trsm_lower_swp<C><<<dim3(L.nf, (m + TRSM_COLS - 1) / TRSM_COLS), TRSM_COLS, 0, st>>>(L, k0, k1, K1, L.ncols,
                                                                                        (const int*)nullptr));
             launch_gemm<C>(L, k1, K1, K1, L.ncols, k0, k1, st, p->d_err, tcp);
           }
@@ -1952,7 +2120,7 @@ void nd_factor_launch(NdPlan* p, const void* alpha64, const void* cint64, const 
         for (int jb = (J1 - 1) / NB; jb >= J0 / NB; --jb) {
           const int j0 = jb * NB, j1 = std::min(j0 + NB, L.smax);
           LS_LAUNCH(f32 ? "nd_trsm_c64" : "nd_trsm_c128", st,
-                    k_trsm_upper<C><<<dim3(L.nf, (m2 + 127) / 128), 128, 0, st>>>(L, j0, j1));
+                    k_trsm_upper<C><<<dim3(L.nf, (m2 + TRSM_COLS - 1) / TRSM_COLS), TRSM_COLS, 0, st>>>(L, j0, j1));
           launch_gemm<C>(L, J0, j0, L.smax, L.ncols, j0, j1, st, p->d_err, tcp);
         }
         launch_gemm<C>(L, 0, J0, L.smax, L.ncols, J0, J1, st, p->d_err, tcp);
@@ -2645,17 +2813,27 @@ __global__ void __launch_bounds__(32 * SMALL_FPC) k_sweep_small(SweepK<float2> S
 }
 
 constexpr int SMALL_MAX_K = 256;
-// the automatic values of the solve-level choices (measured: 2D n = 256 with 16 right-hand
-// sides solves 1.9x faster with neither tensor-core levels nor one-CTA-per-front levels past
-// 64 columns than with the 64-right-hand-side choices; 3D n = 64 with 8 keeps its
-// tensor-core levels)
-int nd_tcs_min_rows(int d, int ng, int v) { return v >= 0 ? v : ((d == 3 || ng >= 2) ? 64 : (1 << 30)); }
-int nd_small_max_k(int ng, int v) { return v >= 0 ? v : (ng >= 2 ? SMALL_MAX_K : 64); }
+// The automatic solve-level choices, per level.
+// Tensor-core levels (from 64 product rows): the level's product has at least 2^25 complex terms;
+// below, its three launches take longer than the one of the CUDA-core sweep (whole solves: 2D
+// n = 128 / 256 / 512 with 21 / 21 / 20 right-hand sides 1.41 / 2.38 / 8.61 ms with tensor-core
+// levels, 1.09 / 1.98 / 7.97 ms without; 3D n = 48 with 8, whose levels are above, 4.43 and 4.71).
+// One-CTA-per-front levels: up to 64 columns; up to 256 with at least two groups of right-hand
+// sides and 512 fronts (fewer leave most SMs without a CTA).
+constexpr double TCS_MIN_TERMS = 33554432.0;
+constexpr int SMALL_MIN_FRONTS = 512;
+static bool tcs_auto(const LevelDev& D, int mode, int ng) {
+  return tcs_rows(D, mode) >= 64 && (double)D.nf * tcs_rows(D, mode) * tcs_k(D, mode) * ng * 16 >= TCS_MIN_TERMS;
+}
+static int small_max_k(const LevelDev& D, int ng, int tune) {
+  if (tune >= 0) return tune;
+  return ng >= 2 && D.nf >= SMALL_MIN_FRONTS ? SMALL_MAX_K : 64;
+}
 
 static bool small_level(const NdPlan* p, int l, int mode, int ng) {
   const LevelDev& D = p->lev[l];
   const int rows = mode == 0 ? D.bmax : D.smax, K = mode == 0 ? D.smax : D.bmax + D.smax;
-  return rows > 0 && rows <= 64 && K > 0 && K <= std::min(SMALL_MAX_K, nd_small_max_k(ng, p->tune.small_max_k));
+  return rows > 0 && rows <= 64 && K > 0 && K <= std::min(SMALL_MAX_K, small_max_k(D, ng, p->tune.small_max_k));
 }
 
 template <int MODE> static void launch_sweep_small(NdPlan* p, int l, float2* T, int ng, cudaStream_t st) {
@@ -2709,8 +2887,9 @@ template <int MODE> static void launch_sweep_small(NdPlan* p, int l, float2* T, 
 static bool tcs_level(const NdPlan* p, int l, int mode, int ng) {
   const LevelDev& D = p->lev[l];
   const int rows = tcs_rows(D, mode);
-  const int min_rows = nd_tcs_min_rows(p->d, ng, mode == 0 ? p->tune.tcs_min_rows : p->tune.tcs_bwd_min_rows);
-  return p->use_tc && tc_enabled() && p->tcs_B && p->tcs_C && rows >= std::max(TCS_MIN_ROWS, min_rows) &&
+  const int tune = mode == 0 ? p->tune.tcs_min_rows : p->tune.tcs_bwd_min_rows;
+  return p->use_tc && tc_enabled() && p->tcs_B && p->tcs_C &&
+         (tune < 0 ? tcs_auto(D, mode, ng) : rows >= std::max(TCS_MIN_ROWS, tune)) &&
          tcs_k(D, mode) >= TC_MIN_K && (size_t)D.nf * tcs_k(D, mode) * ng * 16 <= p->tcs_B_elems &&
          (size_t)D.nf * rows * ng * 16 * tcs_split(D, mode).nsplit <= p->tcs_C_elems;
 }
