@@ -1578,18 +1578,22 @@ __global__ void __launch_bounds__(256) k_gemm(LevelK<C> L, int r0, int r1, int c
     }
     __syncthreads();
   }
+  // all loads before the stores (which the compiler must assume may alias)
+  C old[4][4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int c = cb + ty + 16 * j;
-    if (c >= c1) continue;
+  for (int j = 0; j < 4; ++j)
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int r = rb + tx + 16 * i;
-      if (r >= r1) continue;
-      C& x = A[(size_t)c * fmax + r];
-      x = csub(x, acc[i][j]);
+      const int c = cb + ty + 16 * j, r = rb + tx + 16 * i;
+      if (c < c1 && r < r1) old[i][j] = A[(size_t)c * fmax + r];
     }
-  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int c = cb + ty + 16 * j, r = rb + tx + 16 * i;
+      if (c < c1 && r < r1) A[(size_t)c * fmax + r] = csub(old[i][j], acc[i][j]);
+    }
 }
 
 // One CTA per front (fronts whose own-row block fits in shared memory): extend-add of the

@@ -313,6 +313,14 @@ __global__ void __launch_bounds__(tc::THREADS) k_tc_cgemm(TcArgs a) {
     for (int cc = 0; cc < NT / 2; cc += 16) {
       const int col = half * (NT / 2) + cc;
       uint32_t re[16], im[16];
+      // the entries of C that the product is subtracted from, all loads in flight together (read
+      // and written one after the other they cost a round trip to memory each, 32 in a row)
+      float2 old[EXT ? 1 : 16];
+      if constexpr (!EXT) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          old[j] = rb + m < a.r1 && cb + col + j < a.c1 ? F[(size_t)(cb + col + j) * fmax + rb + m] : make_float2(0.f, 0.f);
+      }
       asm volatile(
           "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
           : "=r"(re[0]), "=r"(re[1]), "=r"(re[2]), "=r"(re[3]), "=r"(re[4]), "=r"(re[5]), "=r"(re[6]), "=r"(re[7]),
@@ -346,11 +354,8 @@ __global__ void __launch_bounds__(tc::THREADS) k_tc_cgemm(TcArgs a) {
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           const int c = cb + col + j;
-          if (c < a.c1) {
-            float2& x = F[(size_t)c * fmax + rb + m];
-            x.x -= __uint_as_float(re[j]);
-            x.y -= __uint_as_float(im[j]);
-          }
+          if (c < a.c1)
+            F[(size_t)c * fmax + rb + m] = make_float2(old[j].x - __uint_as_float(re[j]), old[j].y - __uint_as_float(im[j]));
         }
       }
     }
