@@ -589,41 +589,63 @@ template <typename C> __global__ void k_set_one(C* F, long n_one, const int64_t*
   }
 }
 
-// Schur complements of the children with child index k into their parents' fronts.
-template <typename C> __global__ void __launch_bounds__(256) k_extend_add(LevelK<C> P, LevelK<C> Ch, int k) {
-  const int c = blockIdx.x;
-  if (Ch.kidx[c] != k) return;
-  const int pz = Ch.parent[c];
-  C* Fp = P.F + (size_t)pz * P.fmax * P.ncols;
-  const C* Fc = Ch.F + (size_t)c * Ch.fmax * Ch.ncols;
-  const int* ea = Ch.ea + (size_t)c * Ch.bmax;
-  const int cb = Ch.bmax;
-  const long tot = (long)cb * cb;
-  // four entries per thread: index, child and parent loads in flight before the stores
-  constexpr int B = 4;
-  const long step = (long)gridDim.y * blockDim.x;
-  for (long base = blockIdx.y * (long)blockDim.x + threadIdx.x; base < tot; base += step * B) {
-    C v[B], o[B];
-    long dst[B];
+// Schur complements of both children added into the fronts, front by front: entry (pa, pb) takes the
+// entry of each child whose ring holds both positions (fsrc maps a front position to the children's
+// ring positions), so the front's entries are read and written once and one launch serves a level.
+// grid (fronts, column chunks of cpb columns); shared memory: 2 fmax ints, the children's row of
+// each front row (-1: none).
+constexpr int EA_THREADS = 256;
+template <typename C>
+__global__ void __launch_bounds__(EA_THREADS) k_extend_add(LevelK<C> P, LevelK<C> Ch, const int* __restrict__ fsrc, int cpb) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int* rows = reinterpret_cast<int*>(smem_raw);
+  const int z = blockIdx.x, fmax = P.fmax, cf = Ch.fmax;
+  const int* src = fsrc + (size_t)z * fmax * 2;
+  const C* Fc[2];
+  int base[2];
 #pragma unroll
-    for (int u = 0; u < B; ++u) {
-      const long idx = base + u * step;
-      dst[u] = -1;
-      if (idx < tot) {
-        const int a = (int)(idx % cb), b = (int)(idx / cb);
-        const int pa = ea[a], pb = ea[b];
-        if (pa >= 0 && pb >= 0) {
-          dst[u] = (long)pb * P.fmax + pa;
-          v[u] = Fc[(size_t)(Ch.smax + b) * Ch.fmax + Ch.smax + a];
-        }
+  for (int k = 0; k < 2; ++k) {
+    const int c = P.child[(size_t)z * 2 + k];
+    // fsrc holds c * cf + smax_c + a; ring row a of child c is at Fc[k][.. + a]
+    base[k] = c >= 0 ? c * cf + Ch.smax : 0;
+    Fc[k] = Ch.F + (size_t)(c >= 0 ? c : 0) * cf * Ch.ncols + (size_t)Ch.smax * cf + Ch.smax;
+  }
+  for (int p = threadIdx.x; p < 2 * fmax; p += EA_THREADS) {
+    const int v = __ldg(src + p);  // (row p / 2, child p % 2)
+    rows[p] = v >= 0 ? v - base[p & 1] : -1;
+  }
+  __syncthreads();
+  C* F = P.F + (size_t)z * fmax * P.ncols;
+  const int c0 = blockIdx.y * cpb, c1 = min(fmax, c0 + cpb);
+  // 64 threads down the rows, four columns side by side; four columns per thread with their loads in
+  // flight together
+  constexpr int B = 4, TX = 64, TY = EA_THREADS / TX;
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  for (int pa = tx; pa < fmax; pa += TX) {
+    const int2 a = *reinterpret_cast<const int2*>(rows + 2 * pa);
+    if (a.x < 0 && a.y < 0) continue;
+    const C* s0 = Fc[0] + max(a.x, 0);
+    const C* s1 = Fc[1] + max(a.y, 0);
+    for (int p0 = c0 + ty; p0 < c1; p0 += B * TY) {
+      C o[B], u0[B], u1[B];
+      bool h0[B], h1[B];
+#pragma unroll
+      for (int u = 0; u < B; ++u) {
+        const int pb = p0 + u * TY;
+        const int2 b = pb < c1 ? *reinterpret_cast<const int2*>(rows + 2 * pb) : make_int2(-1, -1);
+        h0[u] = a.x >= 0 && b.x >= 0;
+        h1[u] = a.y >= 0 && b.y >= 0;
+        if (h0[u]) u0[u] = s0[(size_t)b.x * cf];
+        if (h1[u]) u1[u] = s1[(size_t)b.y * cf];
+        if (h0[u] || h1[u]) o[u] = F[(size_t)pb * fmax + pa];
+      }
+#pragma unroll
+      for (int u = 0; u < B; ++u) {
+        if (h0[u]) o[u] = cadd(o[u], u0[u]);
+        if (h1[u]) o[u] = cadd(o[u], u1[u]);
+        if (h0[u] || h1[u]) F[(size_t)(p0 + u * TY) * fmax + pa] = o[u];
       }
     }
-#pragma unroll
-    for (int u = 0; u < B; ++u)
-      if (dst[u] >= 0) o[u] = Fp[dst[u]];
-#pragma unroll
-    for (int u = 0; u < B; ++u)
-      if (dst[u] >= 0) Fp[dst[u]] = cadd(o[u], v[u]);
   }
 }
 
@@ -1755,6 +1777,168 @@ __global__ void __launch_bounds__(256) k_gauss_jordan(LevelK<C> L, LevelK<C> Ch,
   }
 }
 
+// The same elimination with one warp per front, for at most 16 own rows (S = 4, 8 or 16): lane
+// (row r, g) holds row r's columns c = g (mod G), G = 32 / S, in registers, the current block of G
+// columns first (NL columns a lane).  A step is a warp reduction for the pivot, the pivot row's
+// lanes writing their normalised columns to shared memory, and every lane updating its own; no
+// block barrier, and no entry of the block goes through shared memory more than once (the CTA
+// form keeps it there: three barriers and one load and store per entry and step.  2D n = 1024, all levels of up
+// to 16 own rows: 2.47 -> 1.62 ms; 65536 leaf fronts of 16 own and 20 ring rows 1.22 -> 0.76 ms.)
+// The solved rows go to the front and, with ring != 0, to shared memory, from where the ring rows'
+// [S | Y] is formed with a ring row per lane.
+constexpr int GJW_FRONTS = 4;  // warps (fronts) per CTA
+template <typename C> __host__ __device__ constexpr size_t gjw_smem(int S, int nl, int nco, bool ring) {
+  return ((size_t)nl * (32 / S) + (ring ? (size_t)nco * S : 64)) * sizeof(C);  // (64: the child's map)
+}
+// resident CTAs: registers for the values, the ring row and about 30 more
+template <int S, int NL> __host__ __device__ constexpr int gjw_ctas() { return NL > 28 ? 3 : 512 / (2 * NL + (NL < S ? 2 * S : 0) + 40); }
+template <typename C, int S, int NL>
+__global__ void __launch_bounds__(32 * GJW_FRONTS, gjw_ctas<S, NL>()) k_gj_warp(LevelK<C> L, LevelK<C> Ch, int has_child, int* err, int ring) {
+  constexpr int G = 32 / S;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31, wf = threadIdx.x >> 5;
+  const int z = blockIdx.x * GJW_FRONTS + wf;
+  if (z >= L.nf) return;  // (whole warps; no block barriers below)
+  const int s = L.smax, fmax = L.fmax, nc = L.ncols, nco = nc - s;
+  C* prow = reinterpret_cast<C*>(smem_raw + wf * gjw_smem<C>(S, NL, nco, ring != 0));  // normalised pivot row
+  C* B = prow + NL * G;  // [nco][S]: the solved rows of [H | F11^{-1}]
+  C* A = L.F + (size_t)z * fmax * nc;
+  if (has_child) {
+    // extend-add as in k_gauss_jordan
+    int* eas = reinterpret_cast<int*>(B);
+    for (int k = 0; k < 2; ++k) {
+      const int c = L.child[(size_t)z * 2 + k];
+      if (c < 0) continue;
+      const C* __restrict__ Fc = Ch.F + (size_t)c * Ch.fmax * Ch.ncols + (size_t)Ch.smax * Ch.fmax + Ch.smax;
+      const int cb = Ch.bmax, tot = cb * cb;
+      for (int a = lane; a < cb; a += 32) eas[a] = Ch.ea[(size_t)c * cb + a];
+      __syncwarp();
+      for (int base = lane; base < tot; base += 4 * 32) {
+        C v[4], o[4];
+        int dst[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int idx = base + u * 32;
+          dst[u] = -1;
+          if (idx < tot) {
+            const int a = idx % cb, b = idx / cb, pa = eas[a], pb = eas[b];
+            if (pa >= 0 && pb >= 0) {
+              dst[u] = pb * fmax + pa;
+              v[u] = Fc[(size_t)b * Ch.fmax + a];
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (dst[u] >= 0) o[u] = A[dst[u]];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (dst[u] >= 0) A[dst[u]] = cadd(o[u], v[u]);
+      }
+      __syncwarp();
+    }
+  }
+  const int r = lane % S, g = lane / S;
+  C a[NL];
+#pragma unroll
+  for (int l = 0; l < NL; ++l) {
+    const int c = g + G * l;
+    a[l] = r < s && c < nc ? A[(size_t)c * fmax + r] : czero<C>();
+  }
+  bool live = r < s;
+  int jp = r;  // the own row this lane's row solves (its pivot column)
+#pragma unroll 1
+  for (int b = 0; b * G < s; ++b) {
+#pragma unroll
+    for (int g0 = 0; g0 < G; ++g0) {
+      const int j = b * G + g0;
+      if (j < s) {
+        __syncwarp();  // the last step's reads of prow
+        const bool cand = live && g == g0;
+        const unsigned key = cand ? __float_as_uint((float)(fabs(a[0].x) + fabs(a[0].y))) : 0u;
+        const unsigned km = __reduce_max_sync(0xffffffffu, key);
+        const unsigned who = __ballot_sync(0xffffffffu, cand && key == km);  // lowest row on ties
+        const int pl = who ? __ffs(who) - 1 : S * g0, p = pl % S;
+        if (lane == 0 && (km == 0u || who == 0u)) atomicCAS(err, 0, 1);
+        const C m0 = shfl_c(a[0], r + S * g0);  // this row's entry of column j
+        const C dg = shfl_c(a[0], pl);
+        const C inv = pivot_inverse(dg);
+        if (r == p) {
+          live = false;
+          jp = j;
+#pragma unroll
+          for (int l = 0; l < NL; ++l) {
+            a[l] = cmul(a[l], inv);
+            prow[l * G + g] = a[l];
+          }
+        }
+        __syncwarp();
+        const C m = r == p ? czero<C>() : m0;
+        // columns up to j are done with: what the update leaves in them is not used
+        if (g0 < G - 1) {
+#pragma unroll
+          for (int l = 0; l < NL; ++l) a[l] = cfms(a[l], m, prow[l * G + g]);
+        } else {
+#pragma unroll
+          for (int l = 1; l < NL; ++l) a[l - 1] = cfms(a[l], m, prow[l * G + g]);
+        }
+      }
+    }
+  }
+  const int rot = s / G;  // a[l] is column g + G (l + rot)
+  __syncwarp();
+#pragma unroll
+  for (int l = 0; l < NL; ++l) {
+    const int c = g + G * (l + rot);
+    if (c >= s && c < nc) {
+      if (r < s) A[(size_t)c * fmax + jp] = a[l];
+      if (ring) B[(size_t)(c - s) * S + jp] = r < s ? a[l] : czero<C>();
+    }
+  }
+  if (!ring) return;
+  __syncwarp();
+  // ring row i, column c: acc = F - F21 [H | F11^{-1}], four columns at a time
+  const int nb = fmax - s;
+  for (int i0 = 0; i0 < nb; i0 += 32) {
+    const int i = i0 + lane;
+    if (i >= nb) break;
+    C f[S];
+#pragma unroll
+    for (int k = 0; k < S; ++k) f[k] = k < s ? A[(size_t)k * fmax + s + i] : czero<C>();
+    C* row = A + (size_t)s * fmax + s + i;
+    for (int c = 0; c < nco; c += 4) {
+      C acc[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (c + u < nco) acc[u] = row[(size_t)(c + u) * fmax];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (c + u < nco) {
+          const C* bc = B + (size_t)(c + u) * S;
+#pragma unroll
+          for (int k = 0; k < S; ++k) acc[u] = cfms(acc[u], f[k], bc[k]);
+        }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (c + u < nco) row[(size_t)(c + u) * fmax] = acc[u];
+    }
+  }
+}
+
+// Ring rows' [S | Y] = [F22 | 0] - F21 [H | F11^{-1}] of levels with few fronts, one entry per thread:
+// the elimination's own CTA would leave the other SMs idle (FP64, whose two lanes an SM are the
+// bound: all levels of 2D n = 32 0.69 ms with it, 0.38 ms without).
+template <typename C> __global__ void __launch_bounds__(64) k_ring_small(LevelK<C> L) {
+  const int s = L.smax, fmax = L.fmax, b = fmax - s, nco = L.ncols - s;
+  const int t = blockIdx.y * 64 + threadIdx.x;
+  if (t >= b * nco) return;
+  const int i = s + t % b, c = s + t / b;
+  C* A = L.F + (size_t)blockIdx.x * fmax * L.ncols;
+  C acc = A[(size_t)c * fmax + i];
+  for (int k = 0; k < s; ++k) acc = cfms(acc, A[(size_t)k * fmax + i], A[(size_t)c * fmax + k]);
+  A[(size_t)c * fmax + i] = acc;
+}
+
 template <typename C> LevelK<C> level_k(NdPlan* p, int l) {
   const LevelDev& D = p->lev[l];
   LevelK<C> k;
@@ -1878,6 +2062,40 @@ template <typename C> static void launch_gemm(const LevelK<C>& L, int r0, int r1
             k_gemm<C><<<dim3(L.nf, nr * nc), 256, 0, st>>>(L, r0, r1, c0, c1, k0, k1));
 }
 
+// the warp-per-front Gauss-Jordan with room for the level's columns; false if there is none
+template <typename C, int S, int NL>
+static bool launch_gj_warp_n(const LevelK<C>& L, const LevelK<C>& Ch, bool fused_ea, int* err, bool ring, cudaStream_t st) {
+  if ((L.ncols + 32 / S - 1) / (32 / S) > NL) return false;
+  const size_t smem = GJW_FRONTS * gjw_smem<C>(S, NL, L.ncols - L.smax, ring);
+  static std::atomic<bool> attr{false};  // set once per process; repeats are harmless
+  if (!attr.load(std::memory_order_acquire)) {
+    LS_CUDA(cudaFuncSetAttribute(k_gj_warp<C, S, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(GJW_FRONTS * gjw_smem<C>(S, NL, NL * (32 / S), true))));
+    attr.store(true, std::memory_order_release);
+  }
+  LS_LAUNCH(sizeof(C) == 8 ? "nd_gauss_jordan_c64" : "nd_gauss_jordan_c128", st,
+            k_gj_warp<C, S, NL><<<(L.nf + GJW_FRONTS - 1) / GJW_FRONTS, 32 * GJW_FRONTS, smem, st>>>(
+                L, Ch, fused_ea ? 1 : 0, err, ring ? 1 : 0));
+  return true;
+}
+// FP32 levels with at least 256 fronts (below, the CTA form has more threads on each: 128 fronts of
+// 16 own rows 27 against 32 us; in FP64 its more threads hide the latency of the pipe: all levels of
+// 2D n = 32 0.69 against 1.31 ms)
+constexpr int GJW_MIN_FRONTS = 256;
+static bool launch_gj_warp(const LevelK<float2>& L, const LevelK<float2>& Ch, bool ea, int* err, bool ring, cudaStream_t st) {
+  using C = float2;
+  if (L.nf < GJW_MIN_FRONTS || L.smax > 16) return false;
+  if (L.smax <= 4)
+    return launch_gj_warp_n<C, 4, 4>(L, Ch, ea, err, ring, st) || launch_gj_warp_n<C, 4, 8>(L, Ch, ea, err, ring, st);
+  if (L.smax <= 8)
+    return launch_gj_warp_n<C, 8, 8>(L, Ch, ea, err, ring, st) || launch_gj_warp_n<C, 8, 14>(L, Ch, ea, err, ring, st) ||
+           launch_gj_warp_n<C, 8, 20>(L, Ch, ea, err, ring, st);
+  return launch_gj_warp_n<C, 16, 16>(L, Ch, ea, err, ring, st) || launch_gj_warp_n<C, 16, 28>(L, Ch, ea, err, ring, st) ||
+         launch_gj_warp_n<C, 16, 40>(L, Ch, ea, err, ring, st) || launch_gj_warp_n<C, 16, 52>(L, Ch, ea, err, ring, st) ||
+         launch_gj_warp_n<C, 16, 64>(L, Ch, ea, err, ring, st);
+}
+static bool launch_gj_warp(const LevelK<double2>&, const LevelK<double2>&, bool, int*, bool, cudaStream_t) { return false; }
+
 template <typename C> bool nd_prepare(NdPlan* p, cudaStream_t st) { return ensure_buffers(p, sizeof(C), st); }
 
 void nd_set_tensor_cores(NdPlan* p, bool on) { p->use_tc = on; }
@@ -1962,10 +2180,12 @@ void nd_factor_launch(NdPlan* p, const void* alpha64, const void* cint64, const 
   constexpr size_t PANEL_SMEM_MAX = 200 * 1024;
   constexpr int REG_MAX_COLS = 1024;
   constexpr size_t GJ_SMEM_MAX = 160 * 1024;
+  constexpr int EA_FUSED_MIN_FRONTS = 1024, RING_OWN_MIN_FRONTS = 256;
   static std::atomic<bool> attr{false};  // set once per process; repeats are harmless
   if (!attr.load(std::memory_order_acquire)) {
     LS_CUDA(cudaFuncSetAttribute(k_panel<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PANEL_SMEM_MAX));
     LS_CUDA(cudaFuncSetAttribute(k_gauss_jordan<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GJ_SMEM_MAX));
+    LS_CUDA(cudaFuncSetAttribute(k_extend_add<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PANEL_SMEM_MAX));
     attr.store(true, std::memory_order_release);
   }
   bool marked = top_levels == nullptr;
@@ -1989,21 +2209,29 @@ void nd_factor_launch(NdPlan* p, const void* alpha64, const void* cint64, const 
     // n = 256: 1 % faster with the 32-row levels on the register path, 6 % slower with
     // the 8- and 16-row levels there too)
     const bool gj = gjm <= GJ_SMEM_MAX && (L.smax <= p->tune.gj_max_own || L.smax > 32 * reg_rpl_max<C>());
-    const bool fused_ea = gj && has_child && Ch.bmax < 48;
+    // (one warp or CTA per front takes long over its children's entries: it pays where a level has
+    // more fronts than the GPU has room for)
+    const bool fused_ea = gj && has_child && Ch.bmax < 48 && L.nf >= EA_FUSED_MIN_FRONTS;
     if (has_child && !fused_ea) {
-      const long tot = (long)Ch.bmax * Ch.bmax;
-      const unsigned bx = (unsigned)std::max<long>(1, std::min<long>((tot + 1023) / 1024, 64));
-      for (int k = 0; k < 2; ++k)
-        LS_LAUNCH(f32 ? "nd_extend_add_c64" : "nd_extend_add_c128", st,
-                  k_extend_add<C><<<dim3(Ch.nf, bx), 256, 0, st>>>(L, Ch, k));
+      // columns per CTA: about eight CTAs per SM over the level, at least 1 K entries each
+      const long want = std::max<long>(1, 8L * 152 / L.nf);
+      const int cpb = (int)std::max<long>((L.fmax + want - 1) / want, std::min<long>(L.fmax, 1024 / L.fmax + 1));
+      const size_t smem = 2 * (size_t)L.fmax * sizeof(int);
+      LS_LAUNCH(f32 ? "nd_extend_add_c64" : "nd_extend_add_c128", st,
+                k_extend_add<C><<<dim3(L.nf, (L.fmax + cpb - 1) / cpb), EA_THREADS, smem, st>>>(L, Ch, p->lev[l].fsrc, cpb));
     }
     if (gj) {
       // one CTA per front: Gauss-Jordan in shared memory (with the extend-add if fused), and
       // the ring rows' product in the same CTA unless it goes to the tensor cores
       const bool ring_tc = gemm_on_tc<C>(L.bmax, L.smax, tcp);
-      LS_LAUNCH(f32 ? "nd_gauss_jordan_c64" : "nd_gauss_jordan_c128", st,
-                k_gauss_jordan<C><<<L.nf, gj_threads(L.smax, L.ncols), gjm, st>>>(L, Ch, fused_ea ? 1 : 0,
-                                                                                   p->d_err, ring_tc ? 0 : 1));
+      const bool ring_small = !ring_tc && L.nf < RING_OWN_MIN_FRONTS && L.bmax > 0;
+      if (!launch_gj_warp(L, Ch, fused_ea, p->d_err, !ring_tc && !ring_small, st))
+        LS_LAUNCH(f32 ? "nd_gauss_jordan_c64" : "nd_gauss_jordan_c128", st,
+                  k_gauss_jordan<C><<<L.nf, gj_threads(L.smax, L.ncols), gjm, st>>>(L, Ch, fused_ea ? 1 : 0,
+                                                                                     p->d_err, ring_tc || ring_small ? 0 : 1));
+      if (ring_small)
+        LS_LAUNCH(f32 ? "nd_gemm_c64" : "nd_gemm_c128", st,
+                  k_ring_small<C><<<dim3(L.nf, (L.bmax * (L.ncols - L.smax) + 63) / 64), 64, 0, st>>>(L));
       if (ring_tc) launch_gemm<C>(L, L.smax, L.fmax, L.smax, L.ncols, 0, L.smax, st, p->d_err, tcp);
       continue;
     }
