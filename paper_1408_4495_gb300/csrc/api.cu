@@ -378,12 +378,12 @@ template <typename C, typename Cv = double2> void precond_apply(ls_ctx* c, int n
 
 // |[A;B] v - M z|^2 and |[A;B] v|^2 of the first right-hand side of the last preconditioner
 // application (FP32 path), into out[0].x and out[1].x
-void precond_error(ls_ctx* c, const float2* v, const float2* z, double2* partial, double2* out) {
+void precond_error(ls_ctx* c, const float2* v, const float2* z, double2* partial, double2* out, unsigned* cnt) {
   const float2* sv = buf<float2>(c, "pre_r32", (size_t)c->N);  // [A;B] v of that application
   float2* r2 = buf<float2>(c, "pre_est", (size_t)c->N);
   ls::pre_resid(c->d, c->n, 1, v, z, r2, c->alpha32, c->cint64, c->w2m32, c->st);
-  ls::norms2<float2>(r2, c->N, 1, partial, out, 1, c->st);
-  ls::norms2<float2>(sv, c->N, 1, partial, out + 1, 1, c->st);
+  ls::norms2<float2>(r2, c->N, 1, partial, out, 1, cnt, c->st);
+  ls::norms2<float2>(sv, c->N, 1, partial, out + 1, 1, cnt, c->st);
 }
 
 ls_status fail(ls_ctx* c, const Error& e) {
@@ -419,15 +419,17 @@ void solve_impl(ls_ctx* c, int nrhs, const double2* g, double tol, double2* u, l
   CZ* wz = mixed ? buf<CZ>(c, "w32", tot) : nullptr;
   const int nblk = ls::dots_blocks(N);
   double2* partial = buf<double2>(c, "partial", (size_t)nrhs * (R + 2) * nblk);
+  unsigned* cnt = buf<unsigned>(c, "kr_cnt", nrhs);
   double2* hd = buf<double2>(c, "hcol", (size_t)nrhs * (R + 2) * 2);
   double* sd = buf<double>(c, "scale", nrhs);
   ffc* hff = mixed ? buf<ffc>(c, "h_ff", (size_t)nrhs * (R + 2) * 2) : nullptr;
   double2* yd = buf<double2>(c, "ycoef", (size_t)nrhs * R);
   double2* est = mixed ? buf<double2>(c, "pre_err", 2) : nullptr;
 
+  LS_CUDA(cudaMemsetAsync(cnt, 0, nrhs * sizeof(unsigned), c->st));
   LS_CUDA(cudaMemsetAsync(u, 0, tot * sizeof(double2), c->st));
   std::vector<double2> hh((size_t)nrhs * (R + 2) * 2);
-  ls::norms2<double2>(g, N, nrhs, partial, hd, 1, c->st);
+  ls::norms2<double2>(g, N, nrhs, partial, hd, 1, cnt, c->st);
   LS_CUDA(cudaMemcpyAsync(hh.data(), hd, nrhs * sizeof(double2), cudaMemcpyDeviceToHost, c->st));
   LS_CUDA(cudaStreamSynchronize(c->st));
   std::vector<double> gn(nrhs), rn(nrhs);
@@ -494,7 +496,7 @@ void solve_impl(ls_ctx* c, int nrhs, const double2* g, double tol, double2* u, l
                     if (mixed) precond_apply<CZ, float2>(c, nrhs, (const float2*)c->V[k], zk);
                     else precond_apply<CZ>(c, nrhs, c->V[k], zk);
                     if constexpr (sizeof(CZ) == 8)
-                      if (estimate) precond_error(c, (const float2*)c->V[k], zk, partial, est);
+                      if (estimate) precond_error(c, (const float2*)c->V[k], zk, partial, est, cnt);
                     if (mixed) op_apply<CZ>(c, nrhs, zk, wz);
                     else op_apply<double2>(c, nrhs, (const double2*)zk, w);
                     return;
@@ -503,7 +505,7 @@ void solve_impl(ls_ctx* c, int nrhs, const double2* g, double tol, double2* u, l
                     ls::rhs_gather<float2>((const float2*)c->V[k], (float2*)vlive, dlive, nlive, N, c->st);
                     precond_apply<CZ, float2>(c, nlive, (const float2*)vlive, zlive);
                     if constexpr (sizeof(CZ) == 8)
-                      if (estimate) precond_error(c, (const float2*)vlive, zlive, partial, est);
+                      if (estimate) precond_error(c, (const float2*)vlive, zlive, partial, est, cnt);
                   } else {
                     ls::rhs_gather<double2>(c->V[k], vlive, dlive, nlive, N, c->st);
                     precond_apply<CZ>(c, nlive, vlive, zlive);
@@ -529,16 +531,16 @@ void solve_impl(ls_ctx* c, int nrhs, const double2* g, double tol, double2* u, l
         const float2* const* dVf = reinterpret_cast<const float2* const*>(dV);
         float2* wf = reinterpret_cast<float2*>(w);
         ffc* hff2 = hff + (size_t)nrhs * (R + 2);
-        ls::dots_f(dVf, k + 1, (const float2*)wz, N, nrhs, partial, hd, hff, R + 2, c->st);
-        ls::sub_proj_f(dVf, k + 1, (const float2*)wz, wf, hff, R + 2, N, nrhs, partial, nullptr, 0, c->st);
-        ls::dots_f(dVf, k + 1, wf, N, nrhs, partial, hd2, hff2, R + 2, c->st);
-        ls::sub_proj_f(dVf, k + 1, wf, wf, hff2, R + 2, N, nrhs, partial, hd2 + (k + 1), R + 2, c->st);
+        ls::dots_f(dVf, k + 1, (const float2*)wz, N, nrhs, partial, hd, hff, R + 2, cnt, c->st);
+        ls::sub_proj_f(dVf, k + 1, (const float2*)wz, wf, hff, R + 2, N, nrhs, partial, nullptr, 0, cnt, c->st);
+        ls::dots_f(dVf, k + 1, wf, N, nrhs, partial, hd2, hff2, R + 2, cnt, c->st);
+        ls::sub_proj_f(dVf, k + 1, wf, wf, hff2, R + 2, N, nrhs, partial, hd2 + (k + 1), R + 2, cnt, c->st);
       } else {
-        ls::dots<double2>(dV, k + 1, w, N, nrhs, partial, hd, R + 2, false, c->st);
+        ls::dots<double2>(dV, k + 1, w, N, nrhs, partial, hd, R + 2, cnt, c->st);
         ls::sub_proj<double2>(dV, k + 1, w, w, hd, R + 2, N, nrhs, c->st);
-        ls::dots<double2>(dV, k + 1, w, N, nrhs, partial, hd2, R + 2, false, c->st);
+        ls::dots<double2>(dV, k + 1, w, N, nrhs, partial, hd2, R + 2, cnt, c->st);
         ls::sub_proj<double2>(dV, k + 1, w, w, hd2, R + 2, N, nrhs, c->st);
-        ls::norms2<double2>(w, N, nrhs, partial, hd2 + (k + 1), R + 2, c->st);
+        ls::norms2<double2>(w, N, nrhs, partial, hd2 + (k + 1), R + 2, cnt, c->st);
       }
       LS_CUDA(cudaMemcpyAsync(hh.data(), hd, hh.size() * sizeof(double2), cudaMemcpyDeviceToHost, c->st));
       double2 est_h[2] = {};
@@ -615,7 +617,7 @@ void solve_impl(ls_ctx* c, int nrhs, const double2* g, double tol, double2* u, l
         op_apply<double2>(c, nrhs, u, Au);
         ls::residual(g, Au, r, tot, c->st);
       }
-      ls::norms2<double2>(r, N, nrhs, partial, hd, 1, c->st);
+      ls::norms2<double2>(r, N, nrhs, partial, hd, 1, cnt, c->st);
     });
     LS_CUDA(cudaMemcpyAsync(hh.data(), hd, nrhs * sizeof(double2), cudaMemcpyDeviceToHost, c->st));
     LS_CUDA(cudaStreamSynchronize(c->st));
