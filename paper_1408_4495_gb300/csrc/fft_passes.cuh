@@ -23,6 +23,7 @@
 #include "common.cuh"
 #include "fft_lines.cuh"
 #include "kernels.h"
+#include "pdl.cuh"
 #include "prof.h"
 
 namespace ls {
@@ -113,6 +114,7 @@ __global__ void __launch_bounds__(RowShape<C, L>::NT, RowShape<C, L>::MINB) k_ro
   }
   line_fft<C, L, -1, true, false, SH::WARP, LAY>(v, reinterpret_cast<C*>(smem_raw) + li * LAY::LS,
                                                  static_cast<const C*>(a.tw), t);
+  pdl_trigger_small();
   if (!valid) return;
   C* out = static_cast<C*>(a.out) + line * a.out_ls;
 #pragma unroll
@@ -134,6 +136,7 @@ __global__ void __launch_bounds__(RowShape<C, L>::NT, RowShape<C, L>::MINB) k_ro
   const long line = (long)blockIdx.x * SH::NL + li;
   const bool valid = line < a.lines;
   C v[E];
+  pdl_wait();
   const C* in = static_cast<const C*>(a.in) + line * a.in_ls;
 #pragma unroll
   for (int m = 0; m < E / R1; ++m)
@@ -141,6 +144,7 @@ __global__ void __launch_bounds__(RowShape<C, L>::NT, RowShape<C, L>::MINB) k_ro
     for (int r = 0; r < R1; ++r) v[m * R1 + r] = valid ? in[t + m * T + r * (L / R1)] : czero_l<C>();
   line_fft<C, L, 1, false, true, SH::WARP, LAY>(v, reinterpret_cast<C*>(smem_raw) + li * LAY::LS,
                                                 static_cast<const C*>(a.tw), t);
+  pdl_trigger_small();
   if (!valid) return;
   // the added and subtracted entries of a butterfly are loaded together, before any store (the
   // output may be one of them)
@@ -211,11 +215,12 @@ __global__ void __launch_bounds__(ColShape<C, L>::NT, ColShape<C, L>::MINB) k_co
   const int tiles = (int)(a.inner / TC);
   const long o = blockIdx.x / tiles;
   const int c0 = (int)(blockIdx.x - o * tiles) * TC + c;
-  const C* __restrict__ in = static_cast<const C*>(a.in) + o * a.in_os + c0;
+  const C* in = static_cast<const C*>(a.in) + o * a.in_os + c0;
   C* out = static_cast<C*>(a.out) + o * a.out_os + c0;
   const C* tw = static_cast<const C*>(a.tw);
   C* s = reinterpret_cast<C*>(smem_raw) + c * LAY::LS;
   C v[E];
+  pdl_wait();
   if constexpr (MODE != 1) {
 #pragma unroll
     for (int m = 0; m < E / F1; ++m)
@@ -229,6 +234,7 @@ __global__ void __launch_bounds__(ColShape<C, L>::NT, ColShape<C, L>::MINB) k_co
       for (int r = 0; r < FL; ++r) v[m * FL + r] = in[(t + m * T + r * (L / FL)) * a.in_es];
   }
   if constexpr (MODE == 0) {
+    pdl_trigger_small();
 #pragma unroll
     for (int m = 0; m < E / FL; ++m)
 #pragma unroll
@@ -259,6 +265,7 @@ __global__ void __launch_bounds__(ColShape<C, L>::NT, ColShape<C, L>::MINB) k_co
   }
   if constexpr (MODE != 0) {
     line_fft<C, L, 1, false, true, SH::WARP, LAY>(v, s, tw, t);
+    pdl_trigger_small();
 #pragma unroll
     for (int m = 0; m < E / F1; ++m)
 #pragma unroll
@@ -290,7 +297,7 @@ template <typename C, int L, bool OUT64> void launch_row_inv(const RowPassArgs& 
   pass_smem(k_row_inv<C, L, OUT64>, SH::SMEM, attr);
   static const std::string cls = std::string("fft_row_inv_") + arith_tag<C>();
   const long blocks = (a.lines + SH::NL - 1) / SH::NL;
-  if (blocks > 0) LS_LAUNCH(cls.c_str(), st, k_row_inv<C, L, OUT64><<<(unsigned)blocks, SH::NT, SH::SMEM, st>>>(a));
+  if (blocks > 0) LS_LAUNCH(cls.c_str(), st, launch_pdl(k_row_inv<C, L, OUT64>, (unsigned)blocks, SH::NT, SH::SMEM, st, a));
 }
 // the forms that the operator uses: FP32 vectors in FP32 or FP64, FP64 in FP64, float-float in FP64
 template <typename C, int L> void launch_row_L(int sign, const RowPassArgs& a, cudaStream_t st) {
@@ -320,7 +327,7 @@ template <typename C, int L, int MODE> void launch_col_L(const ColPassArgs& a, c
   static const std::string cls =
       std::string(MODE == 0 ? "fft_col_fwd_" : MODE == 1 ? "fft_col_inv_" : "fft_col_sym_") + arith_tag<C>();
   const long blocks = a.inner / SH::TC * a.outer;
-  if (blocks > 0) LS_LAUNCH(cls.c_str(), st, k_col_pass<C, L, MODE><<<(unsigned)blocks, SH::NT, SH::SMEM, st>>>(a));
+  if (blocks > 0) LS_LAUNCH(cls.c_str(), st, launch_pdl(k_col_pass<C, L, MODE>, (unsigned)blocks, SH::NT, SH::SMEM, st, a));
 }
 
 #define LS_FOR_L(X) X(16) X(32) X(48) X(64) X(96) X(128) X(256) X(512) X(1024) X(2048) X(4096)

@@ -8,6 +8,7 @@
 #include "common.cuh"
 #include "ffloat.cuh"
 #include "krylov.h"
+#include "pdl.cuh"
 #include "prof.h"
 
 namespace ls {
@@ -76,7 +77,7 @@ __device__ __forceinline__ void reduce_partials(const double2* partial, int nv, 
 
 // partial[(rhs * nv + j) * nblk + blk] = sum over the block's chunk of conj(V_j) w
 template <typename Cw>
-__global__ void __launch_bounds__(KT) k_dots(const double2* const* __restrict__ V, int nv, const Cw* __restrict__ w,
+__global__ void __launch_bounds__(KT) k_dots(const double2* const* __restrict__ V, int nv, const Cw* w,
                                              long N, double2* partial, int nblk, unsigned* cnt, double2* out,
                                              int ostride) {
   __shared__ double2 sh[KT / 32];
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(KT) k_dots(const double2* const* __restrict__ 
   const long chunk = (N + nblk - 1) / nblk;
   const long i0 = blk * chunk, i1 = min(N, i0 + chunk);
   const Cw* wr = w + (size_t)rhs * N;
+  pdl_enter();
   for (int j = 0; j < nv; ++j) {
     const double2* vr = V[j] + (size_t)rhs * N;
     double2 acc = make_double2(0, 0);
@@ -96,9 +98,10 @@ __global__ void __launch_bounds__(KT) k_dots(const double2* const* __restrict__ 
 
 // wout = win - sum_j V_j h[rhs][j]
 template <typename Cw>
-__global__ void k_sub_proj(const double2* const* __restrict__ V, int nv, const Cw* __restrict__ win, double2* wout,
-                           const double2* __restrict__ h, int hstride, long N, int nrhs) {
+__global__ void k_sub_proj(const double2* const* __restrict__ V, int nv, const Cw* win, double2* wout,
+                           const double2* h, int hstride, long N, int nrhs) {
   const long tot = N * nrhs;
+  pdl_enter();
   for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < tot; idx += (long)gridDim.x * blockDim.x) {
     const long rhs = idx / N;
     double2 acc = to64(win[idx]);
@@ -110,7 +113,7 @@ __global__ void k_sub_proj(const double2* const* __restrict__ V, int nv, const C
 
 // partial[rhs * nblk + blk] = sum |w|^2 over the chunk (as the .x of a double2)
 template <typename Cw>
-__global__ void __launch_bounds__(KT) k_norm2(const Cw* __restrict__ w, long N, double2* partial, int nblk, unsigned* cnt,
+__global__ void __launch_bounds__(KT) k_norm2(const Cw* w, long N, double2* partial, int nblk, unsigned* cnt,
                                               double2* out, int ostride) {
   __shared__ double2 sh[KT / 32];
   const int rhs = blockIdx.y, blk = blockIdx.x;
@@ -118,6 +121,7 @@ __global__ void __launch_bounds__(KT) k_norm2(const Cw* __restrict__ w, long N, 
   const long i0 = blk * chunk, i1 = min(N, i0 + chunk);
   const Cw* wr = w + (size_t)rhs * N;
   double2 acc = make_double2(0, 0);
+  pdl_enter();
   for (long i = i0 + threadIdx.x; i < i1; i += KT) {
     const double2 v = to64(wr[i]);
     acc.x += v.x * v.x + v.y * v.y;
@@ -182,19 +186,21 @@ void dots(const double2* const* V, int nv, const Cw* w, long N, int nrhs, double
           unsigned* cnt, cudaStream_t st) {
   const int nblk = dots_blocks(N);
   LS_LAUNCH("kr_dots", st,
-            k_dots<Cw><<<dim3(nblk, nrhs), KT, 0, st>>>(V, nv, w, N, partial, nblk, cnt, out, ostride));
+            launch_pdl(k_dots<Cw>, dim3(nblk, nrhs), KT, 0, st, V, nv, w, N, partial, nblk, cnt, out, ostride));
 }
 
 template <typename Cw>
 void sub_proj(const double2* const* V, int nv, const Cw* win, double2* wout, const double2* h, int hstride, long N,
               int nrhs, cudaStream_t st) {
-  LS_LAUNCH("kr_sub_proj", st, k_sub_proj<Cw><<<grid_for(N * nrhs), 256, 0, st>>>(V, nv, win, wout, h, hstride, N, nrhs));
+  LS_LAUNCH("kr_sub_proj", st,
+            launch_pdl(k_sub_proj<Cw>, grid_for(N * nrhs), 256, 0, st, V, nv, win, wout, h, hstride, N, nrhs));
 }
 
 template <typename Cw>
 void norms2(const Cw* w, long N, int nrhs, double2* partial, double2* out, int ostride, unsigned* cnt, cudaStream_t st) {
   const int nblk = dots_blocks(N);
-  LS_LAUNCH("kr_norm2", st, k_norm2<Cw><<<dim3(nblk, nrhs), KT, 0, st>>>(w, N, partial, nblk, cnt, out, ostride));
+  LS_LAUNCH("kr_norm2", st,
+            launch_pdl(k_norm2<Cw>, dim3(nblk, nrhs), KT, 0, st, w, N, partial, nblk, cnt, out, ostride));
 }
 
 void scale(const double2* w, double2* out, const double* s, long N, int nrhs, cudaStream_t st) {
@@ -313,7 +319,7 @@ constexpr int RUN = 4;  // elements per thread summed in FP32 before a float-flo
 // component of that size along V_j in the projected vector, which CGS2's second pass
 // removes; the Arnoldi relation holds with the coefficients as computed, because the
 // projection itself (k_sub_proj_f) runs in float-float.
-__global__ void __launch_bounds__(KT) k_dots_f(const float2* const* __restrict__ V, int nv, const float2* __restrict__ w,
+__global__ void __launch_bounds__(KT) k_dots_f(const float2* const* __restrict__ V, int nv, const float2* w,
                                                long N, double2* partial, int nblk, unsigned* cnt, double2* out,
                                                ffc* outf, int ostride) {
   __shared__ double2 sh[KT / 32];
@@ -321,6 +327,7 @@ __global__ void __launch_bounds__(KT) k_dots_f(const float2* const* __restrict__
   const long chunk = (N + nblk - 1) / nblk;
   const long i0 = blk * chunk, i1 = min(N, i0 + chunk);
   const size_t base = (size_t)rhs * N;
+  pdl_enter();
   for (int jg = 0; jg < nv; jg += JB) {
     const int nj = min(JB, nv - jg);
     ffc acc[JB];
@@ -378,7 +385,7 @@ __global__ void __launch_bounds__(KT) k_dots_f(const float2* const* __restrict__
 constexpr int SP_MAXV = 64;
 template <bool NORM>
 __global__ void __launch_bounds__(KT) k_sub_proj_f(const float2* const* __restrict__ V, int nv, const float2* win,
-                                                   float2* wout, const ffc* __restrict__ hf, int hstride, long N,
+                                                   float2* wout, const ffc* hf, int hstride, long N,
                                                    double2* partial, int nblk, unsigned* cnt, double2* norm_out,
                                                    int ostride) {
   __shared__ double2 sh[KT / 32];
@@ -390,6 +397,7 @@ __global__ void __launch_bounds__(KT) k_sub_proj_f(const float2* const* __restri
   const size_t base = (size_t)rhs * N;
   const ffc* hr = hf + (size_t)rhs * hstride;
   const bool staged = nv <= SP_MAXV;
+  pdl_enter();
   if (staged)
     for (int j = threadIdx.x; j < nv; j += KT) {
       hs[j] = hr[j];
@@ -532,7 +540,7 @@ void dots_f(const float2* const* V, int nv, const float2* w, long N, int nrhs, d
             ffc* outf, int ostride, unsigned* cnt, cudaStream_t st) {
   const int nblk = dots_blocks(N);
   LS_LAUNCH("kr_dots", st,
-            k_dots_f<<<dim3(nblk, nrhs), KT, 0, st>>>(V, nv, w, N, partial, nblk, cnt, out, outf, ostride));
+            launch_pdl(k_dots_f, dim3(nblk, nrhs), KT, 0, st, V, nv, w, N, partial, nblk, cnt, out, outf, ostride));
 }
 
 void sub_proj_f(const float2* const* V, int nv, const float2* win, float2* wout, const ffc* hf, int hstride, long N,
@@ -540,11 +548,11 @@ void sub_proj_f(const float2* const* V, int nv, const float2* win, float2* wout,
   const int nblk = dots_blocks(N);
   if (norm_out)
     LS_LAUNCH("kr_sub_proj", st,
-              k_sub_proj_f<true><<<dim3(nblk, nrhs), KT, 0, st>>>(V, nv, win, wout, hf, hstride, N, partial, nblk, cnt,
+              launch_pdl(k_sub_proj_f<true>, dim3(nblk, nrhs), KT, 0, st, V, nv, win, wout, hf, hstride, N, partial, nblk, cnt,
                                                                   norm_out, ostride));
   else
     LS_LAUNCH("kr_sub_proj", st,
-              k_sub_proj_f<false><<<dim3(nblk, nrhs), KT, 0, st>>>(V, nv, win, wout, hf, hstride, N, partial, nblk, cnt,
+              launch_pdl(k_sub_proj_f<false>, dim3(nblk, nrhs), KT, 0, st, V, nv, win, wout, hf, hstride, N, partial, nblk, cnt,
                                                                    nullptr, 0));
 }
 

@@ -48,6 +48,7 @@
 #include "alloc.h"
 #include "common.cuh"
 #include "kernels.h"
+#include "pdl.cuh"
 #include "prof.h"
 
 namespace ls {
@@ -2395,8 +2396,6 @@ template <typename P> __device__ __forceinline__ P pzero() {
   return p;
 }
 
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
 // asynchronous global -> shared copy of one element; a row outside the tile is zero-filled
 template <int B> __device__ __forceinline__ void cp_async_elem(void* dst, const void* src, bool valid) {
@@ -2718,7 +2717,7 @@ template <typename C, int RC, int TR, int MODE> __global__ void __launch_bounds_
 }
 
 // r[rhs][N] -> T[group][N][RC] (right-hand sides past nr are zero)
-template <typename C, int RC> __global__ void __launch_bounds__(256) k_items_in(const C* __restrict__ r, C* T, int nr, long N) {
+template <typename C, int RC> __global__ void __launch_bounds__(256) k_items_in(const C* r, C* T, int nr, long N) {
   constexpr int TP = 512 / RC;
   __shared__ C s[RC][TP + 1];
   pdl_wait();
@@ -2741,7 +2740,7 @@ template <typename C, int RC> __global__ void __launch_bounds__(256) k_items_in(
 
 // T[group][N][RC] -> x[rhs][N] for the nr right-hand sides (ACC: x += T)
 template <typename C, int RC, bool ACC>
-__global__ void __launch_bounds__(256) k_items_out(const C* T, C* __restrict__ x, int nr, long N) {
+__global__ void __launch_bounds__(256) k_items_out(const C* T, C* x, int nr, long N) {
   constexpr int TP = 512 / RC;
   __shared__ C s[RC][TP + 1];
   pdl_wait();
@@ -2763,22 +2762,6 @@ __global__ void __launch_bounds__(256) k_items_out(const C* T, C* __restrict__ x
       else x[(size_t)rhs * N + i] = s[j][ii];
     }
   }
-}
-
-// launch as a programmatic dependent of the previous kernel in the stream
-template <typename... KArgs, typename... Args>
-static void launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  LS_CUDA(cudaLaunchKernelEx(&cfg, kern, args...));
 }
 
 template <typename C, int RC, int TR, int MODE>

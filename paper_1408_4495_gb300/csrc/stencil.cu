@@ -10,6 +10,7 @@
 #include "common.cuh"
 #include "ffloat.cuh"
 #include "kernels.h"
+#include "pdl.cuh"
 #include "prof.h"
 
 namespace ls {
@@ -25,6 +26,7 @@ __global__ void __launch_bounds__(256) k_stencil(int n, int nrhs, const Cin* __r
                                                  long rs_i, long rs_r, const Cout* __restrict__ alpha) {
   constexpr int P3 = D == 2 ? 9 : 27;
   __shared__ Cout sa[PT ? 1 : P3 * P3];
+  pdl_trigger_small();
   if constexpr (!PT) {
     for (int i = threadIdx.x; i < P3 * P3; i += blockDim.x) sa[i] = alpha[i];
     __syncthreads();
@@ -116,6 +118,7 @@ __global__ void __launch_bounds__(256, 3) k_stencil2_roll(int n, int nrhs, int R
                                                        const double2* __restrict__ cint, const float* __restrict__ w2m) {
   __shared__ float2 sa[81];
   __shared__ float2 sc[9];
+  pdl_trigger_small();
   for (int i = threadIdx.x; i < 81; i += blockDim.x) sa[i] = alpha[i];
   if constexpr (RESID) {
     for (int i = threadIdx.x; i < 9; i += blockDim.x) sc[i] = make_float2((float)cint[i].x, (float)cint[i].y);
@@ -190,6 +193,7 @@ __global__ void __launch_bounds__(256, 3) k_stencil2_items(int n, int nrhs, int 
                                                            const double2* __restrict__ cint,
                                                            const float* __restrict__ w2m) {
   constexpr int CW = 256 / RC;
+  pdl_trigger_small();
   __shared__ float2 sa[81];
   __shared__ float2 sc[9];
   __shared__ float2 tile[2][CW * (RC + 1)];
