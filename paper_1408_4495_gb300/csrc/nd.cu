@@ -755,7 +755,7 @@ __global__ void __launch_bounds__(512) k_panel(LevelK<C> L, int k0, int k1, int*
 // values of W columns (or rows) live in registers, the current one first, and every step moves
 // them down by one as it updates them.  A fully unrolled triangle does less arithmetic, but its
 // straight-line code (40 KB and more, run once per launch) waits for instruction fetches most of
-// the time: TRSMTIMES
+// the time: all solves of a factorization 11.9 -> 9.6 ms at 3-D n = 48, 8.7 -> 5.5 at 2-D n = 1024
 template <int W, typename F> __device__ __forceinline__ void rolling_steps(int i0, int w, F&& body) {
   const int i1 = min(w, i0 + 8);
 #pragma unroll 1
@@ -2421,7 +2421,8 @@ template <typename C> struct SweepK {
   int nsplit;        // column ranges per row tile; their partial sums are added in range
                      // order by the CTA that finishes last
   int ksz;           // columns per range
-  int kv;            // items of the vector operand held in shared memory at once
+  int kv;            // items of the vector operand held in shared memory at once; small levels:
+                     // 1 at a leaf level whose w_own stays in T, else 0
   int ng;            // groups of RC right-hand sides: the CTAs of one front's groups are
                      // adjacent in the grid (x = front * ng + group), so that its factor tile
                      // is read from DRAM once and from L2 by the other groups
@@ -2872,28 +2873,55 @@ __global__ void __launch_bounds__(256) k_tcs_scatter(SweepK<float2> S, const flo
 // columns, FP32, 16 right-hand sides per item): one CTA per front, one warp per group of 16
 // right-hand sides (ng warps).  Before the programmatic-dependent wait the CTA stages the
 // front's indices and copies the first SMALL_KCH columns of its factor tile (shared by the
-// groups) into shared memory with cp.async, overlapping the previous level's tail; after it,
-// column chunk by chunk, every warp gathers its group's vector operand (16 right-hand sides
-// per column; index and data loads of four pieces in flight) and accumulates.  Lane l holds
-// row l (and l + 32 when RP = 64) for all 16 right-hand sides, or, when RP = 16, row l & 15
-// for 8 of them (lanes 16-31 the second half).  Forward: rows are the ring rows of Y, the
-// children's ring updates added at the store.
+// groups) into shared memory with cp.async, overlapping the previous level's tail; after it
+// every warp gathers its group's vector operand and, forward, the children's ring updates (one
+// round of loads, four 16-byte pieces per lane in flight, eight lanes on an item), accumulates
+// (lane l: rows l & 15, + 16, .. for eight of the right-hand sides, lanes 16-31 the other eight)
+// and passes its results through shared memory, so that stores run along the items too.
+// The levels move far more bytes than they compute: with the updates read and the results
+// written by the lane that computes the row (16 bytes of each 128-byte item at a time, in a round
+// of loads of its own after the product) the forward sweeps of a solve at 2-D n = 1024 with 64
+// right-hand sides took 2.92, 2.19, 1.53 and 1.20 ms on the four bottom levels, now 2.38, 1.57, 1.17
+// and 0.90 (their bytes at the copy rate: 1.8, 1.2, 0.8, 0.5).  Backward the stores stay with the
+// rows' lanes and the products scalar: packed accumulators and the detour take 72 registers against
+// 48, which cost the leaves 4.70 against 3.36 ms.
+// At the leaves w_own is r_own, which stays in T (leaf: both sweeps of the level run here).
 constexpr int SMALL_FPC = 4;   // warps per CTA at most (groups of 16 of SOLVE_CHUNK)
 constexpr int SMALL_KCH = 64;  // columns of the factor tile and operand staged at once
-// bytes of the CTA's shared memory: factor chunk (RP x KC complex, RP = 16, 32 or 64 rows,
-// KC = min(K, SMALL_KCH) columns), indices (3 K + 2 RP ints, padded to 16 bytes), then ng
-// operand chunks (KC x 16 complex)
+// Fronts from which the updates are gathered ahead of the product: below, the chain of a CTA counts
+// more than the loads in flight over the GPU (solves at n = 64 with 40 right-hand sides 1.315 ms
+// before, 1.303 with every level early, 1.282 with this line; n = 256 with 16 1.706, 1.646, 1.636).
+constexpr int SMALL_EARLY_FRONTS = 512;
+// bytes of the CTA's shared memory: factor chunk (RP x KC complex, RP a multiple of 16 rows,
+// KC = min(K, SMALL_KCH) columns), indices (3 (K + RP) ints, padded to 16 bytes), then per group
+// the operand chunk (KC x 16 complex) and, forward, the updates (RP x 16)
 __host__ __device__ constexpr int small_kc(int K) { return K < SMALL_KCH ? K : SMALL_KCH; }
 __host__ __device__ constexpr size_t small_head_bytes(int K, int rp) {
-  return ((size_t)rp * small_kc(K) * sizeof(float2) + ((size_t)3 * K + 2 * rp) * sizeof(int) + 15) / 16 * 16;
+  return ((size_t)rp * small_kc(K) * sizeof(float2) + (size_t)3 * (K + rp) * sizeof(int) + 15) / 16 * 16;
 }
-__host__ __device__ constexpr size_t small_smem_bytes(int K, int rp, int ng) {
-  return small_head_bytes(K, rp) + (size_t)ng * small_kc(K) * 16 * sizeof(float2);
+__host__ __device__ constexpr int small_group_items(int mode, int K, int rp) { return small_kc(K) + (mode == 0 ? rp : 0); }
+__host__ __device__ constexpr size_t small_smem_bytes(int mode, int K, int rp, int ng) {
+  return small_head_bytes(K, rp) + (size_t)ng * small_group_items(mode, K, rp) * 16 * sizeof(float2);
+}
+// packed pairs (fma.rn.f32x2: one instruction for both components)
+__device__ __forceinline__ unsigned long long dup2(float x) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
 }
 template <int MODE, int RP, bool MULTI>
 __global__ void __launch_bounds__(32 * SMALL_FPC) k_sweep_small(SweepK<float2> S) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int NJ = RP == 16 ? 8 : 16, NRB = RP == 64 ? 2 : 1;
+  constexpr int NRB = RP / 16, NJ = 8;
+  constexpr bool PACK = MODE == 0 && NRB == 1;
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, NT = blockDim.x;
   const int z = blockIdx.x;
   const int smax = S.smax, bmax = S.bmax, fmax = S.fmax;
@@ -2901,8 +2929,12 @@ __global__ void __launch_bounds__(32 * SMALL_FPC) k_sweep_small(SweepK<float2> S
   const int rows = MODE == 0 ? bmax : smax;
   const int kcap = small_kc(K);
   float2* As = reinterpret_cast<float2*>(smem_raw);  // [kcap][RP]
-  int* ix = reinterpret_cast<int*>(As + (size_t)RP * kcap);  // [3 K] item sources, [2 RP] rows
-  float2* vs = reinterpret_cast<float2*>(smem_raw + small_head_bytes(K, RP)) + (size_t)g * kcap * 16;
+  // item sources: forward 3 (grid point, two children's items) for each column, then each row;
+  // backward the grid point of each column (-1: W), then of each row
+  int* ix = reinterpret_cast<int*>(As + (size_t)RP * kcap);
+  float2* vs = reinterpret_cast<float2*>(smem_raw + small_head_bytes(K, RP)) + (size_t)g * small_group_items(MODE, K, RP) * 16;
+  // forward: rows x 16 updates, then results, piece v of row r at r * 8 + (v ^ (r & 7))
+  float4* us = reinterpret_cast<float4*>(vs + (size_t)kcap * 16);
   const float2* A = S.F + (size_t)z * fmax * S.ncols + (size_t)(MODE == 0 ? fmax : smax) * fmax +
                     (MODE == 0 ? smax : 0);
   auto load_chunk = [&](int kc) {
@@ -2913,38 +2945,79 @@ __global__ void __launch_bounds__(32 * SMALL_FPC) k_sweep_small(SweepK<float2> S
     }
     cp_async_commit();
   };
+  const bool leaf = S.kv != 0, child = MODE == 0 && S.nf_c > 0;
+  const bool early = child && S.nf >= SMALL_EARLY_FRONTS;  // the updates are gathered with the operand
   // ---- prologue: static data only
   load_chunk(0);
-  for (int c = threadIdx.x; c < K; c += NT) {
-    if (MODE == 0) {
-      ix[3 * c] = __ldg(S.own + (size_t)z * smax + c);
-      ix[3 * c + 1] = __ldg(S.fsrc + ((size_t)z * fmax + c) * 2);
-      ix[3 * c + 2] = __ldg(S.fsrc + ((size_t)z * fmax + c) * 2 + 1);
-    } else {
-      ix[3 * c] = c < bmax ? __ldg(S.ring + (size_t)z * bmax + c) : -1;
+  if (MODE == 0) {
+    for (int c = threadIdx.x; c < K + rows; c += NT) {
+      ix[3 * c] = c < K ? __ldg(S.own + (size_t)z * smax + c) : -1;
+      ix[3 * c + 1] = child ? __ldg(S.fsrc + ((size_t)z * fmax + c) * 2) : -1;
+      ix[3 * c + 2] = child ? __ldg(S.fsrc + ((size_t)z * fmax + c) * 2 + 1) : -1;
     }
-  }
-  for (int r = threadIdx.x; r < RP; r += NT) {
-    if (MODE == 0) {
-      const bool rv = r < rows;
-      ix[3 * K + 2 * r] = rv ? __ldg(S.fsrc + ((size_t)z * fmax + smax + r) * 2) : -1;
-      ix[3 * K + 2 * r + 1] = rv ? __ldg(S.fsrc + ((size_t)z * fmax + smax + r) * 2 + 1) : -1;
-    } else {
-      ix[3 * K + 2 * r] = r < rows ? __ldg(S.own + (size_t)z * smax + r) : -1;
+  } else {
+    for (int c = threadIdx.x; c < K + rows; c += NT) {
+      const int o = c < K ? c - bmax : c - K;  // own position
+      ix[c] = c < bmax ? __ldg(S.ring + (size_t)z * bmax + c) : c < K && !leaf ? -1 : __ldg(S.own + (size_t)z * smax + o);
     }
   }
   pdl_wait();
   pdl_trigger();
   __syncthreads();  // indices
   const size_t wrow = (size_t)g * S.nf * fmax + (size_t)z * fmax;
-  const size_t cg = (size_t)g * S.nf_c * S.fmax_c;
-  const int row0 = RP == 16 ? (lane & 15) : lane, j0 = RP == 16 ? (lane >> 4) * 8 : 0;
+  const float4* Tg = reinterpret_cast<const float4*>(S.T + (size_t)g * S.N * 16);
+  const float4* Cg = reinterpret_cast<const float4*>(S.Wc + (size_t)g * S.nf_c * S.fmax_c * 16);
+  float4* Wg = reinterpret_cast<float4*>(S.W + wrow * 16);
+  const int row0 = lane & 15, j0 = (lane >> 4) * NJ;
+  constexpr int GB = 4;
+  // items c0 .. c1 of the operand (and, from K on, the updates) to shared memory
+  auto gather = [&](int c0, int c1) {
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int p0 = lane; p0 < (c1 - c0) * 8; p0 += 32 * GB) {
+      float4 x[GB], y[GB], w[GB];
+#pragma unroll
+      for (int u = 0; u < GB; ++u) {
+        const int p = p0 + 32 * u, c = c0 + (p >> 3), v = p & 7;
+        x[u] = y[u] = w[u] = zero;
+        if (p >= (c1 - c0) * 8) continue;
+        if (MODE == 0) {
+          const int pt = ix[3 * c], s0 = ix[3 * c + 1], s1 = ix[3 * c + 2];
+          if (pt >= 0) x[u] = __ldcg(Tg + (size_t)pt * 8 + v);
+          if (s0 >= 0) y[u] = __ldcg(Cg + (size_t)s0 * 8 + v);
+          if (s1 >= 0) w[u] = __ldcg(Cg + (size_t)s1 * 8 + v);
+        } else {
+          const int pt = ix[c];
+          if (pt >= 0) x[u] = __ldcg(Tg + (size_t)pt * 8 + v);
+          else if (c >= bmax && !leaf) x[u] = __ldcg(Wg + (size_t)(c - bmax) * 8 + v);
+          if (c < bmax) x[u] = make_float4(-x[u].x, -x[u].y, -x[u].z, -x[u].w);  // the H columns
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < GB; ++u) {
+        const int p = p0 + 32 * u, c = c0 + (p >> 3), v = p & 7;
+        if (p >= (c1 - c0) * 8) continue;
+        if (MODE == 0) {
+          x[u] = padd(padd(x[u], y[u]), w[u]);
+          if (c >= K) {
+            us[(c - K) * 8 + (v ^ ((c - K) & 7))] = x[u];
+            continue;
+          }
+          if (!leaf) Wg[(size_t)c * 8 + v] = x[u];
+        }
+        reinterpret_cast<float4*>(vs)[p] = x[u];
+      }
+    }
+  };
+  // one row of 16: the products with the factor's real and imaginary parts in packed accumulators
+  // of their own; more rows: complex multiply-adds
+  unsigned long long re[PACK ? NJ : 1], im[PACK ? NJ : 1];
   float2 acc[NRB][NJ];
 #pragma unroll
   for (int b = 0; b < NRB; ++b)
 #pragma unroll
     for (int j = 0; j < NJ; ++j) acc[b][j] = make_float2(0.f, 0.f);
-  constexpr int GB = 4;
+#pragma unroll
+  for (int j = 0; j < (PACK ? NJ : 1); ++j) re[j] = im[j] = 0ull;
   // MULTI: more than one column chunk (K > SMALL_KCH); else the loop runs once
   for (int kc = 0; kc < (MULTI ? K : 1); kc += SMALL_KCH) {
     const int kw = MULTI ? min(SMALL_KCH, K - kc) : K;
@@ -2952,78 +3025,77 @@ __global__ void __launch_bounds__(32 * SMALL_FPC) k_sweep_small(SweepK<float2> S
       __syncthreads();  // every warp is done with the previous chunk
       load_chunk(kc);
     }
-    for (int p0 = lane; p0 < kw * 8; p0 += 32 * GB) {
-      float4 x[GB];
-#pragma unroll
-      for (int u = 0; u < GB; ++u) {
-        const int p = p0 + 32 * u, c = kc + (p >> 3), v = p & 7;
-        x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (p >= kw * 8) continue;
-        if (MODE == 0) {
-          const int pt = ix[3 * c], s0 = ix[3 * c + 1], s1 = ix[3 * c + 2];
-          if (pt >= 0) x[u] = padd(x[u], __ldcg(reinterpret_cast<const float4*>(S.T + ((size_t)g * S.N + pt) * 16) + v));
-          if (s0 >= 0) x[u] = padd(x[u], __ldcg(reinterpret_cast<const float4*>(S.Wc + (cg + s0) * 16) + v));
-          if (s1 >= 0) x[u] = padd(x[u], __ldcg(reinterpret_cast<const float4*>(S.Wc + (cg + s1) * 16) + v));
-        } else if (c < bmax) {
-          const int pt = ix[3 * c];
-          if (pt >= 0) {
-            const float4 t = __ldcg(reinterpret_cast<const float4*>(S.T + ((size_t)g * S.N + pt) * 16) + v);
-            x[u] = make_float4(-t.x, -t.y, -t.z, -t.w);  // the H columns enter with a minus sign
-          }
-        } else {
-          x[u] = __ldcg(reinterpret_cast<const float4*>(S.W + (wrow + c - bmax) * 16) + v);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < GB; ++u) {
-        const int p = p0 + 32 * u, c = kc + (p >> 3), v = p & 7;
-        if (p >= kw * 8) continue;
-        if (MODE == 0) reinterpret_cast<float4*>(S.W + (wrow + c) * 16)[v] = x[u];
-        reinterpret_cast<float4*>(vs)[p] = x[u];
-      }
+    if (MULTI) {
+      gather(kc, kc + kw);
+      if (early && kc == 0) gather(K, K + rows);
+    } else {
+      gather(0, early ? K + rows : K);
     }
     cp_async_wait<0>();
     __syncthreads();  // the factor chunk (every thread's copies) and this warp's operand
 #pragma unroll 4
     for (int k = 0; k < kw; ++k) {
-      const float4* vv = reinterpret_cast<const float4*>(vs + (size_t)k * 16 + j0);
+      const float2* vk = vs + (size_t)k * 16 + j0;
+      if constexpr (PACK) {
+        const float2 a = As[k * RP + row0];
+        const unsigned long long ax = dup2(a.x), ay = dup2(a.y);
 #pragma unroll
-      for (int b = 0; b < NRB; ++b) {
-        const float2 a = As[k * RP + row0 + 32 * b];
+        for (int j = 0; j < NJ; j += 2) {
+          const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(vk + j);
+          fma2(re[j], ax, v.x);
+          fma2(im[j], ay, v.x);
+          fma2(re[j + 1], ax, v.y);
+          fma2(im[j + 1], ay, v.y);
+        }
+      } else {
+        float4 v[NJ / 2];
 #pragma unroll
-        for (int j = 0; j < NJ / 2; ++j) {
-          const float4 v4 = vv[j];
-          acc[b][2 * j] = cfma(acc[b][2 * j], a, make_float2(v4.x, v4.y));
-          acc[b][2 * j + 1] = cfma(acc[b][2 * j + 1], a, make_float2(v4.z, v4.w));
+        for (int j = 0; j < NJ / 2; ++j) v[j] = reinterpret_cast<const float4*>(vk)[j];
+#pragma unroll
+        for (int b = 0; b < NRB; ++b) {
+          const float2 a = As[k * RP + row0 + 16 * b];
+#pragma unroll
+          for (int j = 0; j < NJ / 2; ++j) {
+            acc[b][2 * j] = cfma(acc[b][2 * j], a, make_float2(v[j].x, v[j].y));
+            acc[b][2 * j + 1] = cfma(acc[b][2 * j + 1], a, make_float2(v[j].z, v[j].w));
+          }
         }
       }
     }
   }
+  if constexpr (PACK) {
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      const float2 r = unpack2(re[j]), i = unpack2(im[j]);
+      acc[0][j] = make_float2(r.x - i.y, r.y + i.x);
+    }
+  }
 #pragma unroll
   for (int b = 0; b < NRB; ++b) {
-    const int row = row0 + 32 * b;
+    const int row = row0 + 16 * b;
     if (row >= rows) continue;
-    float2* dst;
-    if (MODE == 0) {
-      const int s0 = ix[3 * K + 2 * row], s1 = ix[3 * K + 2 * row + 1];
+    const int pt = MODE == 1 ? ix[K + row] : 0;
+    if (MODE == 1 && pt < 0) continue;
+    const int s0 = child && !early ? ix[3 * (K + row) + 1] : -1, s1 = child && !early ? ix[3 * (K + row) + 2] : -1;
 #pragma unroll
-      for (int j = 0; j < NJ; j += 2) {
-        float4 x = make_float4(acc[b][j].x, acc[b][j].y, acc[b][j + 1].x, acc[b][j + 1].y);
-        if (s0 >= 0) x = padd(x, __ldcg(reinterpret_cast<const float4*>(S.Wc + (cg + s0) * 16 + j0 + j)));
-        if (s1 >= 0) x = padd(x, __ldcg(reinterpret_cast<const float4*>(S.Wc + (cg + s1) * 16 + j0 + j)));
-        acc[b][j] = make_float2(x.x, x.y);
-        acc[b][j + 1] = make_float2(x.z, x.w);
+    for (int j = 0; j < NJ; j += 2) {
+      float4 x = make_float4(acc[b][j].x, acc[b][j].y, acc[b][j + 1].x, acc[b][j + 1].y);
+      if (MODE == 0) {
+        float4* o = us + row * 8 + (((j0 + j) / 2) ^ (row & 7));
+        if (early) x = padd(x, *o);
+        if (s0 >= 0) x = padd(x, __ldcg(Cg + (size_t)s0 * 8 + (j0 + j) / 2));
+        if (s1 >= 0) x = padd(x, __ldcg(Cg + (size_t)s1 * 8 + (j0 + j) / 2));
+        *o = x;
+      } else {
+        reinterpret_cast<float4*>(S.T + ((size_t)g * S.N + pt) * 16)[(j0 + j) / 2] = x;
       }
-      dst = S.W + (wrow + smax + row) * 16 + j0;
-    } else {
-      const int pt = ix[3 * K + 2 * row];
-      if (pt < 0) continue;
-      dst = S.T + ((size_t)g * S.N + pt) * 16 + j0;
     }
-#pragma unroll
-    for (int j = 0; j < NJ; j += 2)
-      reinterpret_cast<float4*>(dst)[j / 2] =
-          make_float4(acc[b][j].x, acc[b][j].y, acc[b][j + 1].x, acc[b][j + 1].y);
+  }
+  if (MODE == 1) return;
+  __syncwarp();
+  for (int p = lane; p < rows * 8; p += 32) {
+    const int r = p >> 3, v = p & 7;
+    Wg[(size_t)smax * 8 + p] = us[r * 8 + (v ^ (r & 7))];
   }
 }
 
@@ -3074,28 +3146,32 @@ template <int MODE> static void launch_sweep_small(NdPlan* p, int l, float2* T, 
   S.N = p->N;
   const int K = MODE == 0 ? D.smax : D.bmax + D.smax;
   const int rows = MODE == 0 ? D.bmax : D.smax;
-  const int rp = rows > 32 ? 64 : (rows > 16 ? 32 : 16);
-  const size_t smem = small_smem_bytes(K, rp, ng);
-  const size_t smem_max = small_smem_bytes(SMALL_MAX_K, 64, SMALL_FPC);
-  static std::atomic<bool> attr{false};  // set once per process; repeats are harmless
-  if (!attr.load(std::memory_order_acquire)) {
-    LS_CUDA(cudaFuncSetAttribute(k_sweep_small<MODE, 16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
-    LS_CUDA(cudaFuncSetAttribute(k_sweep_small<MODE, 32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
-    LS_CUDA(cudaFuncSetAttribute(k_sweep_small<MODE, 64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
-    LS_CUDA(cudaFuncSetAttribute(k_sweep_small<MODE, 16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
-    LS_CUDA(cudaFuncSetAttribute(k_sweep_small<MODE, 32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
-    LS_CUDA(cudaFuncSetAttribute(k_sweep_small<MODE, 64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
-    attr.store(true, std::memory_order_release);
-  }
+  S.kv = !has_child && small_level(p, l, 0, ng) && small_level(p, l, 1, ng);
+  const int rp = (rows + 15) / 16 * 16;
+  const size_t smem = small_smem_bytes(MODE, K, rp, ng);
   // one CTA per front, one warp per group
   const dim3 grid((unsigned)D.nf), block(32 * ng);
   const char* cls = MODE == 0 ? "nd_fwd_c64" : "nd_bwd_c64";
   const bool multi = K > SMALL_KCH;
-#define LS_SMALL(RP_, M_) LS_LAUNCH(cls, st, launch_pdl(k_sweep_small<MODE, RP_, M_>, grid, block, smem, st, S))
-  if (rp == 64) { if (multi) LS_SMALL(64, true); else LS_SMALL(64, false); }
-  else if (rp == 32) { if (multi) LS_SMALL(32, true); else LS_SMALL(32, false); }
-  else { if (multi) LS_SMALL(16, true); else LS_SMALL(16, false); }
-#undef LS_SMALL
+  auto launch = [&](auto rpc, auto mc) {
+    constexpr int RP = decltype(rpc)::value;
+    constexpr bool MULTI = decltype(mc)::value;
+    static std::atomic<bool> attr{false};  // set once per process; repeats are harmless
+    if (!attr.load(std::memory_order_acquire)) {
+      LS_CUDA(cudaFuncSetAttribute(k_sweep_small<MODE, RP, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)small_smem_bytes(MODE, SMALL_MAX_K, RP, SMALL_FPC)));
+      attr.store(true, std::memory_order_release);
+    }
+    LS_LAUNCH(cls, st, launch_pdl(k_sweep_small<MODE, RP, MULTI>, grid, block, smem, st, S));
+  };
+  auto by_chunks = [&](auto rpc) {
+    if (multi) launch(rpc, std::true_type());
+    else launch(rpc, std::false_type());
+  };
+  if (rp == 64) by_chunks(std::integral_constant<int, 64>());
+  else if (rp == 48) by_chunks(std::integral_constant<int, 48>());
+  else if (rp == 32) by_chunks(std::integral_constant<int, 32>());
+  else by_chunks(std::integral_constant<int, 16>());
 }
 
 // whether level l's sweep product of this mode runs on the tensor cores
