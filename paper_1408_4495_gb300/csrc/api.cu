@@ -26,6 +26,7 @@
 
 #include "alloc.h"
 #include "common.cuh"
+#include "far_plan.h"
 #include "kernels.h"
 #include "ffloat.cuh"
 #include "krylov.h"

@@ -20,6 +20,7 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "far_plan.h"
 #include "kernels.h"
 #include "prof.h"
 
@@ -27,7 +28,6 @@ namespace ls {
 
 namespace {
 
-constexpr int FL = 16;        // grid lines (last axis) per CTA
 constexpr int FK = 16;        // point pairs of a line per chunk
 constexpr int FTHREADS = 128;  // 8 groups of two lines x 16 direction groups
 
@@ -174,21 +174,7 @@ __global__ void __launch_bounds__(256) k_far_reduce(int d, int nobs, int tiles, 
   out[(size_t)r * ostride + k] = make_double2(-hd * v.x, -hd * v.y);
 }
 
-int far_tiles(int d, int n) { return (int)(((d == 2 ? (long)n : (long)n * n) + FL - 1) / FL); }
-
-// directions per pass: the partial sums of one pass stay below about 256 MB
-int far_chunk(int d, int n, int nrhs, int nobs) {
-  const long most = (16L << 20) / ((long)nrhs * far_tiles(d, n)) / 64 * 64;
-  return (int)std::min<long>(nobs, std::max<long>(64, most));
-}
-
 }  // namespace
-
-// complex entries of the tables and the partial sums
-size_t far_scratch_elems(int d, int n, int nrhs, int nobs) {
-  const size_t ko = far_chunk(d, n, nrhs, nobs);
-  return (size_t)nrhs * d * n + (size_t)(d - 1) * n * ko + (size_t)(n / 2) * ko + (size_t)nrhs * far_tiles(d, n) * ko;
-}
 
 template <int D, int TN>
 static void launch_far_sum(int n, int nrhs, int nobs, int tiles, const double2* us, const double* w, const FarTabs& tab,
@@ -203,8 +189,8 @@ void far_field(int d, int n, int nrhs, int nobs, const double2* us, const double
   const double2 cd = d == 2 ? make_double2(cos(M_PI / 4) / sqrt(8 * M_PI * omega), sin(M_PI / 4) / sqrt(8 * M_PI * omega))
                             : make_double2(1.0 / (4 * M_PI), 0.0);
   const int tiles = far_tiles(d, n), chunk = far_chunk(d, n, nrhs, nobs);
-  for (int kc = 0; kc < nobs; kc += chunk) {
-    const int ko = std::min(chunk, nobs - kc);
+  for (long kc = 0; kc < nobs; kc += chunk) {
+    const int ko = (int)std::min<long>(chunk, nobs - kc);
     const double* ob = obs + (size_t)kc * d;
     const size_t n0 = (size_t)nrhs * d * n, n1 = (size_t)(d - 1) * n * ko, n2 = (size_t)(n / 2) * ko;
     double2 *inc = scratch, *outer = inc + n0, *cs = outer + n1, *partial = cs + n2;

@@ -91,10 +91,10 @@ void build_kernel_table(int d, int n, double omega, double h, double2* ktq, cuda
 // Sec. 5: g_r = q_r K delta_{p_r} / h^d for nrhs point sources (pts: nrhs x d grid indices;
 // q: nrhs complex strengths or null for 1), from the quadrant table ktq.
 // far-field pattern u_inf(theta_k; r) of the scattered fields us (nrhs x N) of the plane waves
-// dirs (nrhs x d) in the directions obs (nobs x d); out: nrhs x nobs
+// dirs (nrhs x d) in the directions obs (nobs x d); out: nrhs x nobs; scratch: tables and partial
+// sums, far_scratch_elems entries (far_plan.h)
 void far_field(int d, int n, int nrhs, int nobs, const double2* us, const double* dirs, const double* obs,
                const double* w, double omega, double h, double2* out, double2* scratch, cudaStream_t st);
-size_t far_scratch_elems(int d, int n, int nrhs, int nobs);  // scratch: tables and partial sums
 void point_source(int d, int n, int nrhs, const int* pts, const double2* q, const double2* ktq, double h, double2* g,
                   cudaStream_t st);
 // the symbol's quadrant (fft_symbol.cu); work: (2n)^d entries, tw: symbol_twiddles(2n) on the device

@@ -112,3 +112,32 @@ def test_far_field_tile_edges(LS, d, n, nrhs, nobs):
         ut = O.plane_wave(n, d, omega, dirs[r]) + us[r]
         ref = O.far_field(n, d, omega, m, ut, obs[list(pick)])
         assert np.max(np.abs(F[r][list(pick)] - ref)) < 1e-12 * np.max(np.abs(ref))
+
+
+def _many_directions(LS, n, nobs):
+    """Far field of one wave in nobs directions, a short list repeated: every direction's value must
+    be the short call's to the rounding of the sums, whatever pass and tile it falls in.  Returns the
+    device memory that the long call took."""
+    torch = pytest.importorskip("torch")
+    m, period = medium(2, n, 4), 97
+    short = torch.tensor(obs_dirs(2, period, 5), device="cuda")
+    obs = short.repeat(-(-nobs // period), 1)[:nobs].contiguous()
+    dirs = torch.tensor(obs_dirs(2, 1, 9), device="cuda")
+    rng = np.random.default_rng(1)
+    us = torch.tensor(rng.standard_normal((1, n, n)) + 1j * rng.standard_normal((1, n, n)), device="cuda")
+    out = torch.empty((1, nobs), dtype=torch.complex128, device="cuda")
+    with LS.Solver(torch.tensor(m, device="cuda"), 2 * math.pi * n / 8, dim=2, mixed=True) as s:
+        ref = s.far_field(dirs, us, short)[0]
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        s.far_field(dirs, us, obs, out=out)
+        used = free - torch.cuda.mem_get_info()[0]
+    diff = (out[0] - ref.repeat(-(-nobs // period))[:nobs]).abs().max()
+    assert diff < 1e-12 * ref.abs().max()
+    return used
+
+
+def test_far_field_scratch_is_bounded(LS):
+    """200 000 directions at n = 512, nine passes of 20 928 and a shorter one: 256 MB of scratch (and
+    what the allocator rounds up), against 2.6 GB of tables and partial sums at once."""
+    assert _many_directions(LS, 512, 200000) <= 300 << 20
