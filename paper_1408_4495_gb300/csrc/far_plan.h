@@ -15,7 +15,9 @@ inline long far_dir_elems(int d, int n, int nrhs) {
   return (long)nrhs * far_tiles(d, n) + (long)(d - 1) * n + n / 2;
 }
 
-// Directions per pass: their scratch stays below 256 MB (64 directions at least).
+// Directions per pass: their scratch stays below 256 MB (64 directions at least).  A direction takes
+// 24 entries and more on every grid, so a pass has at most 43 690 tiles of 16 directions: they fit
+// gridDim.z.
 inline int far_chunk(int d, int n, int nrhs, int nobs) {
   const long most = (16L << 20) / far_dir_elems(d, n, nrhs) / 64 * 64;
   return (int)std::min<long>(nobs, std::max<long>(64, most));

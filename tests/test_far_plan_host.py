@@ -32,7 +32,7 @@ def plans(tmp_path_factory):
     src, exe = tmp / "p.cpp", tmp / "p"
     src.write_text(PROG)
     subprocess.run([cxx, "-std=c++17", "-O2", "-I", CSRC, str(src), "-o", str(exe)], check=True)
-    cases = [(d, n, r, k) for d, ns in ((2, (8, 16, 32, 48, 128, 512, 2048)), (3, (8, 24, 64, 128)))
+    cases = [(d, n, r, k) for d, ns in ((2, (16, 32, 48, 128, 512, 2048)), (3, (8, 24, 64, 128)))
              for n, r, k in itertools.product(ns, (1, 3, 32, 512), (1, 64, 9000, 100000, 1048577, 2147483647))]
     out = subprocess.run([str(exe)], check=True, capture_output=True, text=True,
                          input="\n".join(" ".join(map(str, c)) for c in cases)).stdout
@@ -49,3 +49,7 @@ def test_scratch_is_bounded(plans):
         assert elems >= need
         floor = r * d * n + 64 * ((d - 1) * n + n // 2 + r * tiles)
         assert elems * 16 <= max(floor * 16, (256 << 20) + r * d * n * 16)
+
+
+def test_tiles_fit_the_grid(plans):
+    assert max(-(-chunk // 16) for *_, chunk, _ in plans) <= 65535  # k_far_sum's gridDim.z at 16 directions a CTA

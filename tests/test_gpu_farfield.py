@@ -141,3 +141,8 @@ def test_far_field_scratch_is_bounded(LS):
     """200 000 directions at n = 512, nine passes of 20 928 and a shorter one: 256 MB of scratch (and
     what the allocator rounds up), against 2.6 GB of tables and partial sums at once."""
     assert _many_directions(LS, 512, 200000) <= 300 << 20
+
+
+def test_far_field_more_directions_than_the_grid_is_deep(LS):
+    """More than 65535 tiles of 16 directions, on the smallest grid and for one wave."""
+    _many_directions(LS, 16, 1048577)
