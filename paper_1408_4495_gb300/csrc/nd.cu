@@ -3101,16 +3101,21 @@ __global__ void __launch_bounds__(32 * SMALL_FPC) k_sweep_small(SweepK<float2> S
 
 constexpr int SMALL_MAX_K = 256;
 // The automatic solve-level choices, per level.
-// Tensor-core levels (from 64 product rows): the level's product has at least 2^25 complex terms;
-// below, its three launches take longer than the one of the CUDA-core sweep (whole solves: 2D
+// Tensor-core levels (from 64 product rows): in 3D, and in 2D with at least two groups of right-hand
+// sides, where the level's product has at least 2^25 complex terms; below, its three launches take
+// longer than the one of the CUDA-core sweep (whole solves: 2D
 // n = 128 / 256 / 512 with 21 / 21 / 20 right-hand sides 1.41 / 2.38 / 8.61 ms with tensor-core
 // levels, 1.09 / 1.98 / 7.97 ms without; 3D n = 48 with 8, whose levels are above, 4.43 and 4.71).
+// In 2D the products of one group stay on the CUDA cores at every size: FP32 there, 3xTF32 here, and
+// 16 columns fill a quarter of a tile (n = 1024 with 8 right-hand sides 16.9 ms against 17.6 with every
+// level from 64 rows on the tensor cores, with 16 20.3 / 21.0; n = 2048 with 16 80.9 / 78.2).
 // One-CTA-per-front levels: up to 64 columns; up to 256 with at least two groups of right-hand
 // sides and 512 fronts (fewer leave most SMs without a CTA).
 constexpr double TCS_MIN_TERMS = 33554432.0;
 constexpr int SMALL_MIN_FRONTS = 512;
-static bool tcs_auto(const LevelDev& D, int mode, int ng) {
-  return tcs_rows(D, mode) >= 64 && (double)D.nf * tcs_rows(D, mode) * tcs_k(D, mode) * ng * 16 >= TCS_MIN_TERMS;
+static bool tcs_auto(const LevelDev& D, int d, int mode, int ng) {
+  return (d == 3 || ng >= 2) && tcs_rows(D, mode) >= 64 &&
+         (double)D.nf * tcs_rows(D, mode) * tcs_k(D, mode) * ng * 16 >= TCS_MIN_TERMS;
 }
 static int small_max_k(const LevelDev& D, int ng, int tune) {
   if (tune >= 0) return tune;
@@ -3180,7 +3185,7 @@ static bool tcs_level(const NdPlan* p, int l, int mode, int ng) {
   const int rows = tcs_rows(D, mode);
   const int tune = mode == 0 ? p->tune.tcs_min_rows : p->tune.tcs_bwd_min_rows;
   return p->use_tc && tc_enabled() && p->tcs_B && p->tcs_C &&
-         (tune < 0 ? tcs_auto(D, mode, ng) : rows >= std::max(TCS_MIN_ROWS, tune)) &&
+         (tune < 0 ? tcs_auto(D, p->d, mode, ng) : rows >= std::max(TCS_MIN_ROWS, tune)) &&
          tcs_k(D, mode) >= TC_MIN_K && (size_t)D.nf * tcs_k(D, mode) * ng * 16 <= p->tcs_B_elems &&
          (size_t)D.nf * rows * ng * 16 * tcs_split(D, mode).nsplit <= p->tcs_C_elems;
 }
