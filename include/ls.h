@@ -408,7 +408,7 @@ ls_status ls_profile_stop(char* report, int capacity);
  * forward and backward solve levels (rows of their products, at least 32) run on the tensor
  * cores, and the largest bottom solve level (columns of its product, up to 256; rows up to
  * 64) run one CTA per front.  The last three default to -1, automatic by the level's size:
- * tensor-core levels from 64 rows where the level's product has at least 2^25 complex terms,
+ * tensor-core levels from 64 rows where the level's product has at least 1.4 * 2^25 complex terms,
  * in 2D with more than 16 right-hand sides only;
  * one-CTA-per-front levels up to 64 columns, up to 256 on levels of 512 fronts and more with
  * more than 16 right-hand sides.  A coordinate search

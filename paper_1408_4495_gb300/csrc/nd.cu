@@ -3102,16 +3102,18 @@ __global__ void __launch_bounds__(32 * SMALL_FPC) k_sweep_small(SweepK<float2> S
 constexpr int SMALL_MAX_K = 256;
 // The automatic solve-level choices, per level.
 // Tensor-core levels (from 64 product rows): in 3D, and in 2D with at least two groups of right-hand
-// sides, where the level's product has at least 2^25 complex terms; below, its three launches take
-// longer than the one of the CUDA-core sweep (whole solves: 2D
-// n = 128 / 256 / 512 with 21 / 21 / 20 right-hand sides 1.41 / 2.38 / 8.61 ms with tensor-core
-// levels, 1.09 / 1.98 / 7.97 ms without; 3D n = 48 with 8, whose levels are above, 4.43 and 4.71).
+// sides, where the level's product has at least 1.4 * 2^25 complex terms; below, its three launches
+// take longer than the one of the CUDA-core sweep.  Whole solves with no level / every level from 64
+// rows on the tensor cores: 2D n = 256 with 21 right-hand sides 1.52 / 1.73 ms (terms up to 0.3 * 2^25);
+// n = 512 with 20 7.21 / 7.66, with 32 8.43 / 8.86 (up to 1.25); with 64 15.06 / 15.13, 14.77 with those of
+// 1.5 and more; n = 1024 with 20 29.0 / 27.6, with 32 36.7 / 34.3 (most 2 to 5), with 64 67.1 / 59.1; 3D n = 32 with 8
+// 1.45 / 1.78 (up to 1.05), with 32 2.38 / 2.33; n = 48 with 8 6.08 / 5.73 (most 2.5 to 5), n = 64 with 8 15.0 / 12.2.
 // In 2D the products of one group stay on the CUDA cores at every size: FP32 there, 3xTF32 here, and
-// 16 columns fill a quarter of a tile (n = 1024 with 8 right-hand sides 16.9 ms against 17.6 with every
-// level from 64 rows on the tensor cores, with 16 20.3 / 21.0; n = 2048 with 16 80.9 / 78.2).
+// 16 columns fill a quarter of a tile (n = 1024 with 8 right-hand sides 16.9 / 17.6 ms, with 16 20.3 / 21.0; n = 2048
+// with 16 80.9 / 78.2).
 // One-CTA-per-front levels: up to 64 columns; up to 256 with at least two groups of right-hand
 // sides and 512 fronts (fewer leave most SMs without a CTA).
-constexpr double TCS_MIN_TERMS = 33554432.0;
+constexpr double TCS_MIN_TERMS = 1.4 * 33554432.0;
 constexpr int SMALL_MIN_FRONTS = 512;
 static bool tcs_auto(const LevelDev& D, int d, int mode, int ng) {
   return (d == 3 || ng >= 2) && tcs_rows(D, mode) >= 64 &&

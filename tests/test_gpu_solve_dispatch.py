@@ -19,10 +19,10 @@ def LS():
     return ls
 
 
-@pytest.mark.parametrize("n,nrhs", [(1024, 5), (1024, 16)])
+@pytest.mark.parametrize("n,nrhs", [(1024, 5), (1024, 16), (512, 17), (512, 32)])
 def test_levels_stay_on_the_cuda_cores(LS, n, nrhs):
     """One group of right-hand sides in 2D, where levels exceed the rule's number of terms: FP32 at
-    every level."""
+    every level.  Two groups at n = 512: every level has 0.25 to 1.25 times 2^25 terms."""
     import torch
     m = W.enforce_buffer(W.bumps(n, 2, [-0.2], [0.1], [(0.5, 0.5)]), 2)
     gen = torch.Generator(device="cuda").manual_seed(n)
