@@ -2421,8 +2421,8 @@ template <typename C> struct SweepK {
   int nsplit;        // column ranges per row tile; their partial sums are added in range
                      // order by the CTA that finishes last
   int ksz;           // columns per range
-  int kv;            // items of the vector operand held in shared memory at once; small levels:
-                     // 1 at a leaf level whose w_own stays in T, else 0
+  int kv;            // items of the vector operand held in shared memory at once
+  int leaf;          // small levels: 1 where w_own is r_own and stays in T (sweep_leaf)
   int ng;            // groups of RC right-hand sides: the CTAs of one front's groups are
                      // adjacent in the grid (x = front * ng + group), so that its factor tile
                      // is read from DRAM once and from L2 by the other groups
@@ -2885,7 +2885,7 @@ __global__ void __launch_bounds__(256) k_tcs_scatter(SweepK<float2> S, const flo
 // and 0.90 (their bytes at the copy rate: 1.8, 1.2, 0.8, 0.5).  Backward the stores stay with the
 // rows' lanes and the products scalar: packed accumulators and the detour take 72 registers against
 // 48, which cost the leaves 4.70 against 3.36 ms.
-// At the leaves w_own is r_own, which stays in T (leaf: both sweeps of the level run here).
+// At the leaves w_own is r_own, which stays in T where both sweeps of the level run here (sweep_leaf).
 constexpr int SMALL_FPC = 4;   // warps per CTA at most (groups of 16 of SOLVE_CHUNK)
 constexpr int SMALL_KCH = 64;  // columns of the factor tile and operand staged at once
 // Fronts from which the updates are gathered ahead of the product: below, the chain of a CTA counts
@@ -2945,7 +2945,7 @@ __global__ void __launch_bounds__(32 * SMALL_FPC) k_sweep_small(SweepK<float2> S
     }
     cp_async_commit();
   };
-  const bool leaf = S.kv != 0, child = MODE == 0 && S.nf_c > 0;
+  const bool leaf = S.leaf != 0, child = MODE == 0 && S.nf_c > 0;
   const bool early = child && S.nf >= SMALL_EARLY_FRONTS;  // the updates are gathered with the operand
   // ---- prologue: static data only
   load_chunk(0);
@@ -3130,6 +3130,29 @@ static bool small_level(const NdPlan* p, int l, int mode, int ng) {
   return rows > 0 && rows <= 64 && K > 0 && K <= std::min(SMALL_MAX_K, small_max_k(D, ng, p->tune.small_max_k));
 }
 
+// whether level l's sweep product of this mode runs on the tensor cores
+static bool tcs_level(const NdPlan* p, int l, int mode, int ng) {
+  const LevelDev& D = p->lev[l];
+  const int rows = tcs_rows(D, mode);
+  const int tune = mode == 0 ? p->tune.tcs_min_rows : p->tune.tcs_bwd_min_rows;
+  return p->use_tc && tc_enabled() && p->tcs_B && p->tcs_C &&
+         (tune < 0 ? tcs_auto(D, p->d, mode, ng) : rows >= std::max(TCS_MIN_ROWS, tune)) &&
+         tcs_k(D, mode) >= TC_MIN_K && (size_t)D.nf * tcs_k(D, mode) * ng * 16 <= p->tcs_B_elems &&
+         (size_t)D.nf * rows * ng * 16 * tcs_split(D, mode).nsplit <= p->tcs_C_elems;
+}
+
+// The kernel that runs level l's FP32 sweep of this mode on items of 16 right-hand sides.
+enum SweepForm { SWEEP_TILED, SWEEP_SMALL, SWEEP_TC };
+static SweepForm sweep_form(const NdPlan* p, int l, int mode, int ng) {
+  return tcs_level(p, l, mode, ng) ? SWEEP_TC : small_level(p, l, mode, ng) ? SWEEP_SMALL : SWEEP_TILED;
+}
+// w_own of a leaf level is r_own, which T holds until the level's own backward sweep writes x there:
+// k_sweep_small neither writes it to W nor reads it from there where it runs both sweeps (the other
+// forms always do both).
+static bool sweep_leaf(const NdPlan* p, int l, int ng) {
+  return l + 1 == (int)p->lev.size() && sweep_form(p, l, 0, ng) == SWEEP_SMALL && sweep_form(p, l, 1, ng) == SWEEP_SMALL;
+}
+
 template <int MODE> static void launch_sweep_small(NdPlan* p, int l, float2* T, int ng, cudaStream_t st) {
   const LevelDev& D = p->lev[l];
   const int depth = (int)p->lev.size();
@@ -3153,7 +3176,7 @@ template <int MODE> static void launch_sweep_small(NdPlan* p, int l, float2* T, 
   S.N = p->N;
   const int K = MODE == 0 ? D.smax : D.bmax + D.smax;
   const int rows = MODE == 0 ? D.bmax : D.smax;
-  S.kv = !has_child && small_level(p, l, 0, ng) && small_level(p, l, 1, ng);
+  S.leaf = sweep_leaf(p, l, ng);
   const int rp = (rows + 15) / 16 * 16;
   const size_t smem = small_smem_bytes(MODE, K, rp, ng);
   // one CTA per front, one warp per group
@@ -3179,17 +3202,6 @@ template <int MODE> static void launch_sweep_small(NdPlan* p, int l, float2* T, 
   else if (rp == 48) by_chunks(std::integral_constant<int, 48>());
   else if (rp == 32) by_chunks(std::integral_constant<int, 32>());
   else by_chunks(std::integral_constant<int, 16>());
-}
-
-// whether level l's sweep product of this mode runs on the tensor cores
-static bool tcs_level(const NdPlan* p, int l, int mode, int ng) {
-  const LevelDev& D = p->lev[l];
-  const int rows = tcs_rows(D, mode);
-  const int tune = mode == 0 ? p->tune.tcs_min_rows : p->tune.tcs_bwd_min_rows;
-  return p->use_tc && tc_enabled() && p->tcs_B && p->tcs_C &&
-         (tune < 0 ? tcs_auto(D, p->d, mode, ng) : rows >= std::max(TCS_MIN_ROWS, tune)) &&
-         tcs_k(D, mode) >= TC_MIN_K && (size_t)D.nf * tcs_k(D, mode) * ng * 16 <= p->tcs_B_elems &&
-         (size_t)D.nf * rows * ng * 16 * tcs_split(D, mode).nsplit <= p->tcs_C_elems;
 }
 
 template <int MODE> static void launch_sweep_tc(NdPlan* p, int l, float2* T, int ng, cudaStream_t st) {
@@ -3230,14 +3242,10 @@ template <int MODE> static void launch_sweep_tc(NdPlan* p, int l, float2* T, int
 
 template <typename C, int RC, int MODE> static void launch_sweep(NdPlan* p, int l, C* T, int ng, cudaStream_t st) {
   if constexpr (sizeof(C) == 8 && RC == 16) {
-    if (tcs_level(p, l, MODE, ng)) {
-      launch_sweep_tc<MODE>(p, l, reinterpret_cast<float2*>(T), ng, st);
-      return;
-    }
-    if (small_level(p, l, MODE, ng)) {
-      launch_sweep_small<MODE>(p, l, reinterpret_cast<float2*>(T), ng, st);
-      return;
-    }
+    const SweepForm form = sweep_form(p, l, MODE, ng);
+    if (form == SWEEP_TC) launch_sweep_tc<MODE>(p, l, reinterpret_cast<float2*>(T), ng, st);
+    if (form == SWEEP_SMALL) launch_sweep_small<MODE>(p, l, reinterpret_cast<float2*>(T), ng, st);
+    if (form != SWEEP_TILED) return;
   }
   const SweepPlan q = sweep_plan(p->lev[l], MODE, ng, std::min(std::max(p->tune.sweep_ctas, 1), SWEEP_CTAS_MAX));
   if (q.K <= 0) return;
