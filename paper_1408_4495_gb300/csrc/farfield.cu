@@ -22,6 +22,7 @@
 #include "common.cuh"
 #include "far_plan.h"
 #include "kernels.h"
+#include "pdl.cuh"
 #include "prof.h"
 
 namespace ls {
@@ -41,6 +42,7 @@ __global__ void k_far_tables(int d, int n, int nrhs, int nobs, const double* __r
                              const double* __restrict__ obs, double omega, double h, double2* __restrict__ inc,
                              double2* __restrict__ outer, double2* __restrict__ cs) {
   const long n0 = (long)nrhs * d * n, n1 = (long)(d - 1) * n * nobs, n2 = (long)(n / 2) * nobs;
+  pdl_trigger_small();
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n0 + n1 + n2; t += (long)gridDim.x * blockDim.x) {
     double sn, cn;
     if (t < n0) {
@@ -82,6 +84,7 @@ __global__ void __launch_bounds__(FTHREADS) k_far_sum(int n, int nobs, int tiles
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int q = 0; q < TN; ++q) acc[i][q] = make_double2(0.0, 0.0);
+  pdl_enter();
   for (int j0 = 0; j0 < n / 2; j0 += FK) {
     int any = 0;
 #pragma unroll
@@ -154,13 +157,14 @@ __global__ void __launch_bounds__(FTHREADS) k_far_sum(int n, int nobs, int tiles
 }
 
 // out[r][k] = -h^d c_d e^{-i omega theta_{d-1} / 2} * sum over the tiles (8 segments, in order)
-__global__ void __launch_bounds__(256) k_far_reduce(int d, int nobs, int tiles, const double2* __restrict__ partial,
+__global__ void __launch_bounds__(256) k_far_reduce(int d, int nobs, int tiles, const double2* partial,
                                                     const double* __restrict__ obs, double omega, double hd, double2 cd,
                                                     double2* __restrict__ out, int ostride) {
   __shared__ double2 red[8][32];
   const int r = blockIdx.y, lane = threadIdx.x & 31, seg = threadIdx.x >> 5, k = blockIdx.x * 32 + lane;
   const int per = (tiles + 7) / 8, t1 = min(tiles, (seg + 1) * per);
   double2 s = make_double2(0.0, 0.0);
+  pdl_wait();
   if (k < nobs)
     for (int t = seg * per; t < t1; ++t) s = cadd(s, partial[((size_t)r * tiles + t) * nobs + k]);
   red[seg][lane] = s;
@@ -180,8 +184,8 @@ template <int D, int TN>
 static void launch_far_sum(int n, int nrhs, int nobs, int tiles, const double2* us, const double* w, const FarTabs& tab,
                            double2* partial, cudaStream_t st) {
   LS_LAUNCH("far_field", st,
-            k_far_sum<D, TN><<<dim3(tiles, nrhs, (nobs + 16 * TN - 1) / (16 * TN)), FTHREADS, 0, st>>>(
-                n, nobs, tiles, us, w, tab, partial));
+            launch_pdl(k_far_sum<D, TN>, dim3(tiles, nrhs, (nobs + 16 * TN - 1) / (16 * TN)), FTHREADS, 0, st, n, nobs,
+                       tiles, us, w, tab, partial));
 }
 
 void far_field(int d, int n, int nrhs, int nobs, const double2* us, const double* dirs, const double* obs,
@@ -198,16 +202,19 @@ void far_field(int d, int n, int nrhs, int nobs, const double2* us, const double
               k_far_tables<<<(unsigned)std::min<size_t>((n0 + n1 + n2 + 127) / 128, 152 * 8), 128, 0, st>>>(
                   d, n, nrhs, ko, dirs, ob, omega, h, inc, outer, cs));
     // directions per CTA: 64, or 32 or 16 where that leaves fewer idle (a smaller tile forms v_r
-    // more often: about 10 FP64 operations a point against 2 per direction)
+    // more often: about 10 FP64 operations a point against 2 per direction) or SMs without a CTA (one
+    // wave, 64 directions: 2D n = 32 61 -> 42 us a call with the overlapped launches below, n = 128 122 ->
+    // 65, n = 512 311 -> 140; the single launch of a block per wave and direction took 52, 144, 1485)
     const FarTabs tab{inc, outer, cs};
     const int pad64 = (ko + 63) / 64 * 64, pad32 = (ko + 31) / 32 * 32, pad16 = (ko + 15) / 16 * 16;
-    const int tn = pad16 < pad32 ? 1 : (pad32 < pad64 ? 2 : 4);
+    int tn = pad16 < pad32 ? 1 : (pad32 < pad64 ? 2 : 4);
+    while (tn > 1 && (long)tiles * nrhs * ((ko + 16 * tn - 1) / (16 * tn)) < 152) tn /= 2;
     auto sum = d == 2 ? (tn == 1 ? launch_far_sum<2, 1> : (tn == 2 ? launch_far_sum<2, 2> : launch_far_sum<2, 4>))
                       : (tn == 1 ? launch_far_sum<3, 1> : (tn == 2 ? launch_far_sum<3, 2> : launch_far_sum<3, 4>));
     sum(n, nrhs, ko, tiles, us, w, tab, partial, st);
     LS_LAUNCH("far_field", st,
-              k_far_reduce<<<dim3((ko + 31) / 32, nrhs), 256, 0, st>>>(d, ko, tiles, partial, ob, omega,
-                                                                       d == 2 ? h * h : h * h * h, cd, out + kc, nobs));
+              launch_pdl(k_far_reduce, dim3((ko + 31) / 32, nrhs), 256, 0, st, d, ko, tiles, (const double2*)partial, ob,
+                         omega, d == 2 ? h * h : h * h * h, cd, out + kc, nobs));
   }
 }
 

@@ -30,7 +30,7 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // limit; limits of 304 to 1216 CTAs lie between).
 constexpr unsigned PDL_MAX_CTAS = 152;
 __device__ __forceinline__ void pdl_trigger_small() {
-  if (gridDim.x * gridDim.y <= PDL_MAX_CTAS) pdl_trigger();
+  if (gridDim.x * gridDim.y * gridDim.z <= PDL_MAX_CTAS) pdl_trigger();
 }
 __device__ __forceinline__ void pdl_enter() {
   pdl_wait();

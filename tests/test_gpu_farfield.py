@@ -146,3 +146,18 @@ def test_far_field_scratch_is_bounded(LS):
 def test_far_field_more_directions_than_the_grid_is_deep(LS):
     """More than 65535 tiles of 16 directions, on the smallest grid and for one wave."""
     _many_directions(LS, 16, 1048577)
+
+
+@pytest.mark.parametrize("d,n,nrhs,nobs", [(2, 32, 1, 64), (2, 256, 10, 63), (2, 256, 3, 128), (3, 16, 10, 30), (3, 16, 1, 128)])
+def test_far_field_tiles_of_directions(LS, d, n, nrhs, nobs):
+    """16, 32 and 64 directions a CTA, chosen by the number of CTAs: the bound of the tests above."""
+    omega = 2 * math.pi * n / 8
+    m = medium(d, n, 4)
+    dirs, obs = obs_dirs(d, nrhs, 9), obs_dirs(d, nobs, 5)
+    rng = np.random.default_rng(1)
+    us = rng.standard_normal((nrhs,) + (n,) * d) + 1j * rng.standard_normal((nrhs,) + (n,) * d)
+    with LS.Solver(m, omega, mixed=True) as s:
+        F = s.far_field(dirs, us, obs)
+    for r in range(0, nrhs, 4):
+        ref = O.far_field(n, d, omega, m, O.plane_wave(n, d, omega, dirs[r]) + us[r], obs)
+        assert np.max(np.abs(F[r] - ref)) < 1e-12 * np.max(np.abs(ref))
