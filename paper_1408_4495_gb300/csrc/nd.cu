@@ -619,8 +619,9 @@ __global__ void __launch_bounds__(EA_THREADS) k_extend_add(LevelK<C> P, LevelK<C
   C* F = P.F + (size_t)z * fmax * P.ncols;
   const int c0 = blockIdx.y * cpb, c1 = min(fmax, c0 + cpb);
   // 64 threads down the rows, four columns side by side; four columns per thread with their loads in
-  // flight together
-  constexpr int B = 4, TX = 64, TY = EA_THREADS / TX;
+  // flight together, two in FP64 (84 registers with four: half the warps; all levels of 3D n = 24 0.59 ms
+  // with four, 0.41 with two, 0.37 with half the CTAs as well)
+  constexpr int B = sizeof(C) == 8 ? 4 : 2, TX = 64, TY = EA_THREADS / TX;
   const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
   for (int pa = tx; pa < fmax; pa += TX) {
     const int2 a = *reinterpret_cast<const int2*>(rows + 2 * pa);
@@ -2220,8 +2221,8 @@ void nd_factor_launch(NdPlan* p, const void* alpha64, const void* cint64, const 
     // more fronts than the GPU has room for)
     const bool fused_ea = gj && has_child && Ch.bmax < 48 && L.nf >= EA_FUSED_MIN_FRONTS;
     if (has_child && !fused_ea) {
-      // columns per CTA: about eight CTAs per SM over the level, at least 1 K entries each
-      const long want = std::max<long>(1, 8L * 152 / L.nf);
+      // columns per CTA: about eight CTAs per SM over the level (four in FP64), at least 1 K entries each
+      const long want = std::max<long>(1, (f32 ? 8L : 4L) * 152 / L.nf);
       const int cpb = (int)std::max<long>((L.fmax + want - 1) / want, std::min<long>(L.fmax, 1024 / L.fmax + 1));
       const size_t smem = 2 * (size_t)L.fmax * sizeof(int);
       LS_LAUNCH(f32 ? "nd_extend_add_c64" : "nd_extend_add_c128", st,
