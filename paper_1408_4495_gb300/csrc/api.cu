@@ -123,8 +123,9 @@ std::map<StencilKey, std::pair<std::vector<double2>, std::vector<double2>>> g_st
 
 // host twiddle tables per FFT length (one of eleven), kept for the process
 struct LineTables {
-  std::vector<double2> t64, sym;  // the passes' (16-byte values), the symbol transforms'
-  std::vector<float2> t32;        // the FP32 passes'
+  std::vector<double2> t64;  // the passes' (16-byte values, n64 of them), then the symbol transforms'
+  size_t n64;
+  std::vector<float2> t32;   // the FP32 passes'
 };
 const LineTables& line_tables(int L) {
   static std::mutex mu;
@@ -132,9 +133,11 @@ const LineTables& line_tables(int L) {
   std::lock_guard<std::mutex> lk(mu);
   LineTables& t = cache[L];  // (map nodes stay where they are)
   if (t.t32.empty()) {
-    ls::line_twiddles(L, true, t.t64);
-    ls::symbol_twiddles(L, t.sym);
     std::vector<double2> tp;
+    ls::line_twiddles(L, true, t.t64);
+    t.n64 = t.t64.size();
+    ls::symbol_twiddles(L, tp);
+    t.t64.insert(t.t64.end(), tp.begin(), tp.end());
     ls::line_twiddles(L, false, tp);
     t.t32.resize(tp.size());
     for (size_t q = 0; q < tp.size(); ++q) t.t32[q] = make_float2((float)tp[q].x, (float)tp[q].y);
@@ -831,13 +834,13 @@ static ls_status setup_common(const ls_grid* g, double omega, const double* m, b
     c->w2m32 = dalloc<float>(c->N);
     LS_CUDA(cudaMemcpyAsync(c->w2m64, w64.data(), c->N * sizeof(double), cudaMemcpyHostToDevice, c->st));
     LS_CUDA(cudaMemcpyAsync(c->w2m32, w32.data(), c->N * sizeof(float), cudaMemcpyHostToDevice, c->st));
-    // twiddle tables of the passes: FP32 (8-byte values), FP64 and float-float (16-byte values)
+    // twiddle tables of the passes: FP32 (8-byte values), FP64 and float-float (16-byte values, then
+    // the symbol transforms' factors: one copy)
     const int L = c->L;
     const LineTables& tab = line_tables(L);
-    const std::vector<double2>&t64 = tab.t64, &ts = tab.sym;
-    c->tw64 = dalloc<double2>(t64.size());
+    c->tw64 = dalloc<double2>(tab.t64.size());
     c->tw32 = dalloc<float2>(tab.t32.size());
-    LS_CUDA(cudaMemcpyAsync(c->tw64, t64.data(), t64.size() * sizeof(double2), cudaMemcpyHostToDevice, c->st));
+    LS_CUDA(cudaMemcpyAsync(c->tw64, tab.t64.data(), tab.t64.size() * sizeof(double2), cudaMemcpyHostToDevice, c->st));
     LS_CUDA(cudaMemcpyAsync(c->tw32, tab.t32.data(), tab.t32.size() * sizeof(float2), cudaMemcpyHostToDevice, c->st));
     // Nystrom table quadrant and symbol (Sec. 2.1)
     const long n1 = n + 1;
@@ -864,10 +867,9 @@ static ls_status setup_common(const ls_grid* g, double omega, const double* m, b
     c->plan.w2m64 = c->w2m64;
     {
       const long Ld = c->d == 2 ? (long)L * L : (long)L * L * L;
-      double2* work = dalloc<double2>(Ld + ts.size());  // the transform, then its twiddle table
+      double2* work = dalloc<double2>(Ld);
       try {
-        LS_CUDA(cudaMemcpyAsync(work + Ld, ts.data(), ts.size() * sizeof(double2), cudaMemcpyHostToDevice, c->st));
-        ls::build_symbol(c->d, n, c->ktq, c->sym64, c->sym32, work, work + Ld, c->st);
+        ls::build_symbol(c->d, n, c->ktq, c->sym64, c->sym32, work, c->tw64 + tab.n64, c->st);
         LS_CUDA(cudaStreamSynchronize(c->st));
       } catch (...) {
         ls::dev_free(work);
@@ -878,9 +880,9 @@ static ls_status setup_common(const ls_grid* g, double omega, const double* m, b
     c->plan.sym32 = c->sym32;
     c->plan.sym64 = c->sym64;
     {
-      const size_t ntwf = 2 * t64.size(), nsy = 2 * (size_t)nq;  // FP64 components: one float pair each
+      const size_t ntwf = 2 * tab.n64, nsy = 2 * (size_t)nq;  // FP64 components: one float pair each
       c->ffbuf = dalloc<float2>(ntwf + nsy + (size_t)c->N);
-      ls::to_ffp(c->tw64, c->ffbuf, (long)t64.size(), c->st);
+      ls::to_ffp(c->tw64, c->ffbuf, (long)tab.n64, c->st);
       ls::to_ffp(c->sym64, c->ffbuf + ntwf, nq, c->st);
       ls::to_ff(c->w2m64, c->ffbuf + ntwf + nsy, c->N, c->st);
       c->plan.twff = c->ffbuf;

@@ -101,8 +101,12 @@ template <int L, int NS, int LINES, int NT> __device__ __forceinline__ void sym_
   }
 }
 
+// Eight entries a thread.  Short lines in small CTAs, 8 lines and more each (128 bytes of a strided
+// line's row): a small grid has few lines, and with 256 threads at every length they filled a few SMs
+// only (all passes of 3D n = 16 48.7 -> 36.1 us, n = 24 61.2 -> 38.7, 2D n = 64 40.8 -> 28.5; from 3D n = 64
+// and 2D n = 128 on as before, the GPU is full either way).
 template <int L> struct SymShape {
-  static constexpr int NT = L / 8 > 256 ? L / 8 : 256;
+  static constexpr int NT = L > 2048 ? L / 8 : L >= 256 ? 256 : L >= 96 ? L : L == 48 ? 96 : 64;
   static constexpr int LINES = NT * 8 / L;
 };
 
