@@ -137,7 +137,6 @@ __device__ __forceinline__ double f64_of(float f) {
 }
 // hi + lo of a float-float as FP64: one FP64 add (exact when the pair is normalized)
 __device__ __forceinline__ double ff_to_f64(ff a) { return f64_of(a.hi) + f64_of(a.lo); }
-__device__ __forceinline__ double2 ffc_to_f64(ffc v) { return make_double2(ff_to_f64(v.x), ff_to_f64(v.y)); }
 
 // an FP64 number as a float-float: hi = its leading 24 significant bits (truncated), lo =
 // the next 23 bits (rounded half up), so |x - (hi + lo)| <= 2^-47 |x|; lo is built as an exact

@@ -57,7 +57,7 @@ namespace {
 
 struct Node {
   int lo[3], hi[3];
-  int depth = 0, parent = -1, nchild = 0, slot = -1, kidx = -1;
+  int depth = 0, slot = -1;
   int child[2] = {-1, -1};
   std::vector<int> own, ring;
 };
@@ -65,7 +65,7 @@ struct Node {
 struct LevelDev {
   int nf = 0, smax = 0, bmax = 0, fmax = 0, ncols = 0;
   size_t F_off = 0, W_off = 0;
-  int *own = nullptr, *ring = nullptr, *child = nullptr, *parent = nullptr, *kidx = nullptr, *ea = nullptr;
+  int *own = nullptr, *ring = nullptr, *child = nullptr, *ea = nullptr;
   int* piv = nullptr;
   int* fsrc = nullptr;  // per front position: the two children's W items that add into it (-1: none)
 };
@@ -74,7 +74,7 @@ template <typename C> struct LevelK {
   C* F;
   C* W;
   int nf, smax, bmax, fmax, ncols;
-  const int *own, *ring, *child, *parent, *kidx, *ea;
+  const int *own, *ring, *child, *ea;
   int* piv;
 };
 
@@ -123,7 +123,7 @@ struct NdHost {
   long N = 0;
   std::vector<LevelDev> lev;  // shapes and offsets; pointers are set per context
   struct Off {
-    size_t own, ring, child, parent, kidx, ea, piv, fsrc;
+    size_t own, ring, child, ea, piv, fsrc;
   };
   std::vector<Off> off;
   size_t asm_off_o = 0, asm_row_o = 0, asm_t_o = 0, one_off_o = 0, err_o = 0;
@@ -164,13 +164,7 @@ void build_tree(TreeBuild* p, int leaf_max) {
     Node& nd = p->nodes.back();
     for (int a = 0; a < 3; ++a) { nd.lo[a] = it.lo[a]; nd.hi[a] = it.hi[a]; }
     nd.depth = it.depth;
-    nd.parent = it.parent;
-    nd.kidx = it.kidx;
-    if (it.parent >= 0) {
-      Node& par = p->nodes[it.parent];
-      par.child[it.kidx] = id;
-      par.nchild = std::max(par.nchild, it.kidx + 1);
-    }
+    if (it.parent >= 0) p->nodes[it.parent].child[it.kidx] = id;
     int size[3], vol = 1, ax = 0;
     for (int a = 0; a < 3; ++a) { size[a] = it.hi[a] - it.lo[a]; vol *= size[a]; }
     for (int a = 1; a < d; ++a)
@@ -289,14 +283,12 @@ std::shared_ptr<NdHost> host_symbolic(int d, int n) {
       else { c[2] = g % n_; c[1] = (g / n_) % n_; c[0] = g / (n_ * n_); }
     };
     auto flat = [&](const int* c) -> int { return d == 2 ? c[0] * n_ + c[1] : (c[0] * n_ + c[1]) * n_ + c[2]; };
-    std::vector<std::vector<int>> l_own(depth), l_ring(depth), l_child(depth), l_parent(depth), l_kidx(depth), l_ea(depth);
+    std::vector<std::vector<int>> l_own(depth), l_ring(depth), l_child(depth), l_ea(depth);
     for (int l = 0; l < depth; ++l) {
       const LevelDev& L = p->lev[l];
       l_own[l].assign((size_t)L.nf * L.smax, -1);
       l_ring[l].assign((size_t)L.nf * L.bmax, -1);
       l_child[l].assign((size_t)L.nf * 2, -1);
-      l_parent[l].assign(L.nf, -1);
-      l_kidx[l].assign(L.nf, -1);
       l_ea[l].assign((size_t)L.nf * L.bmax, -1);
     }
     const int t_lo2 = d == 3 ? -1 : 0, t_hi2 = d == 3 ? 1 : 0;
@@ -313,10 +305,6 @@ std::shared_ptr<NdHost> host_symbolic(int d, int n) {
       for (int q = 0; q < b; ++q) l_ring[l][(size_t)z * L.bmax + q] = nd.ring[q];
       for (int k = 0; k < 2; ++k)
         if (nd.child[k] >= 0) l_child[l][(size_t)z * 2 + k] = T.nodes[nd.child[k]].slot;
-      if (nd.parent >= 0) {
-        l_parent[l][z] = T.nodes[nd.parent].slot;
-        l_kidx[l][z] = nd.kidx;
-      }
       for (int q = 0; q < s; ++q) pos[nd.own[q]] = q;
       for (int q = 0; q < b; ++q) pos[nd.ring[q]] = L.smax + q;
       const size_t base = L.F_off + (size_t)z * L.fmax * L.ncols;
@@ -383,8 +371,6 @@ std::shared_ptr<NdHost> host_symbolic(int d, int n) {
       o.own = put(p->blob, l_own[l]);
       o.ring = put(p->blob, l_ring[l]);
       o.child = put(p->blob, l_child[l]);
-      o.parent = put(p->blob, l_parent[l]);
-      o.kidx = put(p->blob, l_kidx[l]);
       o.ea = put(p->blob, l_ea[l]);
       o.piv = put(p->blob, std::vector<int>((size_t)L.nf * L.smax, 0));
       // forward-solve sources: child k's ring entry a lands at position ea[a] of the parent
@@ -450,8 +436,6 @@ NdPlan* nd_build(int d, int n, cudaStream_t st) {
       L.own = reinterpret_cast<int*>(b + o.own);
       L.ring = reinterpret_cast<int*>(b + o.ring);
       L.child = reinterpret_cast<int*>(b + o.child);
-      L.parent = reinterpret_cast<int*>(b + o.parent);
-      L.kidx = reinterpret_cast<int*>(b + o.kidx);
       L.ea = reinterpret_cast<int*>(b + o.ea);
       L.piv = reinterpret_cast<int*>(b + o.piv);
       L.fsrc = reinterpret_cast<int*>(b + o.fsrc);
@@ -1953,7 +1937,7 @@ template <typename C> LevelK<C> level_k(NdPlan* p, int l) {
   k.F = reinterpret_cast<C*>(p->F) + D.F_off;
   k.W = reinterpret_cast<C*>(p->W) + D.W_off;
   k.nf = D.nf; k.smax = D.smax; k.bmax = D.bmax; k.fmax = D.fmax; k.ncols = D.ncols;
-  k.own = D.own; k.ring = D.ring; k.child = D.child; k.parent = D.parent; k.kidx = D.kidx; k.ea = D.ea;
+  k.own = D.own; k.ring = D.ring; k.child = D.child; k.ea = D.ea;
   k.piv = D.piv;
   return k;
 }
@@ -2093,13 +2077,11 @@ constexpr int GJW_MIN_FRONTS = 256;
 static bool launch_gj_warp(const LevelK<float2>& L, const LevelK<float2>& Ch, bool ea, int* err, bool ring, cudaStream_t st) {
   using C = float2;
   if (L.nf < GJW_MIN_FRONTS || L.smax > 16) return false;
-  if (L.smax <= 4)
-    return launch_gj_warp_n<C, 4, 4>(L, Ch, ea, err, ring, st) || launch_gj_warp_n<C, 4, 8>(L, Ch, ea, err, ring, st);
+  // the widths of the grids' levels: 4 own rows with 24 ring rows; 8 with 32 and 48; 16 with 16, 64 and 96
+  if (L.smax <= 4) return launch_gj_warp_n<C, 4, 4>(L, Ch, ea, err, ring, st);
   if (L.smax <= 8)
-    return launch_gj_warp_n<C, 8, 8>(L, Ch, ea, err, ring, st) || launch_gj_warp_n<C, 8, 14>(L, Ch, ea, err, ring, st) ||
-           launch_gj_warp_n<C, 8, 20>(L, Ch, ea, err, ring, st);
-  return launch_gj_warp_n<C, 16, 16>(L, Ch, ea, err, ring, st) || launch_gj_warp_n<C, 16, 28>(L, Ch, ea, err, ring, st) ||
-         launch_gj_warp_n<C, 16, 40>(L, Ch, ea, err, ring, st) || launch_gj_warp_n<C, 16, 52>(L, Ch, ea, err, ring, st) ||
+    return launch_gj_warp_n<C, 8, 14>(L, Ch, ea, err, ring, st) || launch_gj_warp_n<C, 8, 20>(L, Ch, ea, err, ring, st);
+  return launch_gj_warp_n<C, 16, 28>(L, Ch, ea, err, ring, st) || launch_gj_warp_n<C, 16, 52>(L, Ch, ea, err, ring, st) ||
          launch_gj_warp_n<C, 16, 64>(L, Ch, ea, err, ring, st);
 }
 static bool launch_gj_warp(const LevelK<double2>&, const LevelK<double2>&, bool, int*, bool, cudaStream_t) { return false; }
