@@ -375,7 +375,8 @@ typedef struct {
   double solve_bytes;      /* bytes of factor read by one forward + backward solve */
   /* bytes moved by one forward sweep (leaves to root) and one backward sweep of the solve,
    * split into the factor blocks read once per sweep and the vector traffic per
-   * right-hand side (gathers, children's updates, front vectors), padded shapes */
+   * right-hand side (gathers, children's updates, front vectors) of the tiled sweeps, padded
+   * shapes (the one-CTA-per-front kernel writes less at the leaves) */
   double fwd_factor_bytes, fwd_bytes_per_rhs;
   double bwd_factor_bytes, bwd_bytes_per_rhs;
 } ls_nd_stats;

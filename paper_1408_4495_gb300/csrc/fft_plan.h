@@ -1,16 +1,14 @@
-// Radix plan of the Stockham line transforms and the layout of the FP32 passes' twiddle
-// table, shared by the passes (device) and the table's construction (host).
+// Radix plan of the symbol's full-length line transforms (fft_symbol.cu, setup only) and the layout of
+// their twiddle table, shared by the kernels (device) and the table's construction (host).  The
+// operator's passes have a plan of their own (fft_lines.h).
 //
-// A line of length L (2^k or 3 * 2^k) is transformed by passes of radix 8 while the remaining
+// A line of length L (2^k or 3 * 2^k) is transformed by Stockham passes of radix 8 while the remaining
 // length is a multiple of 8, then 4 or 2, then 3.  The pass that starts from sub-transforms
 // of length NS (NS > 1) multiplies entry r of butterfly k (0 <= k < NS, 0 <= r < R) by
-// w^{r k}, w = exp(-2 pi i / (NS R)) (conjugated in the inverse transform).  The FP32 table
-// holds these factors pass after pass, butterfly after butterfly: pass NS at
-// tw_pass_offset(L, NS), butterfly k's R factors (r = 0 included) at k * R from there, so
-// that a butterfly reads one contiguous, 16-byte aligned run (sum over the passes of NS * R
-// < 2 L entries).  The FP64 and float-float passes index the L-entry table exp(-2 pi i m / L)
-// at m = r k L / (NS R) instead: with 16-byte entries the per-butterfly runs spread one load
-// instruction of a warp over more cache lines than that table's neighbouring entries do.
+// w^{r k}, w = exp(-2 pi i / (NS R)).  The table holds these factors (FP64) pass after pass, butterfly
+// after butterfly: pass NS at tw_pass_offset(L, NS), butterfly k's R factors (r = 0 included) at k * R
+// from there, so that a butterfly reads one contiguous run (sum over the passes of NS * R < 2 L
+// entries).
 #pragma once
 
 #if defined(__CUDACC__)

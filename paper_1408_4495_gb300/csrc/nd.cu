@@ -253,6 +253,7 @@ std::shared_ptr<NdHost> host_symbolic(int d, int n) {
       cm += (double)L.bmax * L.smax * (L.ncols - L.smax);
       flops += 8.0 * cm * L.nf;
       solve_entries += (double)L.nf * ((double)L.smax * L.smax + 2.0 * L.smax * L.bmax);
+      // (of the tiled sweeps: k_sweep_small does not write the own part at the leaves)
       // forward: Y (bmax x smax) once; per right-hand side: r at the own points, the front
       // vector written (fmax); backward: [H | F11^-1] (smax x (bmax + smax)) once; per
       // right-hand side: x at the ring points, w_own, x written at the own points
@@ -2200,7 +2201,9 @@ void nd_factor_launch(NdPlan* p, const void* alpha64, const void* cint64, const 
     // the 8- and 16-row levels there too)
     const bool gj = gjm <= GJ_SMEM_MAX && (L.smax <= p->tune.gj_max_own || L.smax > 32 * reg_rpl_max<C>());
     // (one warp or CTA per front takes long over its children's entries: it pays where a level has
-    // more fronts than the GPU has room for)
+    // more fronts than the GPU has room for.  FP32 factorizations with the line at 1 / 256 / 1024 fronts / none
+    // fused: 2D n = 64 309 / 286 / 287 / 287 us, n = 128 563 / 551 / 544 / 546, n = 512 4146 / 4148 / 4144 / 4200, n = 1024
+    // 14.98 / 14.97 / 14.98 / 15.24 ms)
     const bool fused_ea = gj && has_child && Ch.bmax < 48 && L.nf >= EA_FUSED_MIN_FRONTS;
     if (has_child && !fused_ea) {
       // columns per CTA: about eight CTAs per SM over the level (four in FP64), at least 1 K entries each
@@ -2212,7 +2215,10 @@ void nd_factor_launch(NdPlan* p, const void* alpha64, const void* cint64, const 
     }
     if (gj) {
       // one CTA per front: Gauss-Jordan in shared memory (with the extend-add if fused), and
-      // the ring rows' product in the same CTA unless it goes to the tensor cores
+      // the ring rows' product in the same CTA unless it goes to the tensor cores or the level has
+      // too few fronts to fill the GPU (factorizations with the product always in the CTA / the line at
+      // 256 / at 2048 fronts: FP64 2D n = 32 772 / 492 / 492 us, n = 128 4.41 / 3.98 / 3.92 ms, 3D n = 16 8.78 / 8.37 /
+      // 8.37; FP32 2D n = 32 231 / 167 / 164 us, n = 128 578 / 544 / 542, 3D n = 16 913 / 903 / 906, n = 32 7.26 / 7.25 / 7.26 ms)
       const bool ring_tc = gemm_on_tc<C>(L.bmax, L.smax, tcp);
       const bool ring_small = !ring_tc && L.nf < RING_OWN_MIN_FRONTS && L.bmax > 0;
       if (!launch_gj_warp(L, Ch, fused_ea, p->d_err, !ring_tc && !ring_small, st))
@@ -3101,7 +3107,10 @@ constexpr int SMALL_MAX_K = 256;
 // 16 columns fill a quarter of a tile (n = 1024 with 8 right-hand sides 16.9 / 17.6 ms, with 16 20.3 / 21.0; n = 2048
 // with 16 80.9 / 78.2).
 // One-CTA-per-front levels: up to 64 columns; up to 256 with at least two groups of right-hand
-// sides and 512 fronts (fewer leave most SMs without a CTA).
+// sides and 512 fronts (on fewer, the tiled sweep's split of a front's rows and columns over CTAs
+// finishes earlier; applications with the line at 128 / 512 / 2048 fronts: 2D n = 256 with 64 right-hand
+// sides 584 / 560 / 559 us, n = 512 with 20 1003 / 957 / 948, n = 1024 with 64 6.42 / 6.42 / 6.46 ms, 3D n = 32 with 64
+// 1.02 / 1.00 / 1.02, n = 48 with 64 3.09 / 3.07 / 3.15).
 constexpr double TCS_MIN_TERMS = 1.4 * 33554432.0;
 constexpr int SMALL_MIN_FRONTS = 512;
 static bool tcs_auto(const LevelDev& D, int d, int mode, int ng) {
