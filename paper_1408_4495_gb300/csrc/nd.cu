@@ -1783,8 +1783,13 @@ constexpr int GJW_FRONTS = 4;  // warps (fronts) per CTA
 template <typename C> __host__ __device__ constexpr size_t gjw_smem(int S, int nl, int nco, bool ring) {
   return ((size_t)nl * (32 / S) + (ring ? (size_t)nco * S : 64)) * sizeof(C);  // (64: the child's map)
 }
-// resident CTAs: registers for the values, the ring row and about 30 more
-template <int S, int NL> __host__ __device__ constexpr int gjw_ctas() { return NL > 28 ? 3 : 512 / (2 * NL + (NL < S ? 2 * S : 0) + 40); }
+// Resident CTAs asked for: an SM's registers hold 512 for each of a CTA's threads, of which a CTA takes 2 NL for
+// the values, 2 S for the ring row where the values do not cover it and about 40 for the rest.  The two wide
+// forms take two CTAs' worth: at three they spill up to 1 KB a thread (all levels of 2D n = 512 0.475 -> 0.442
+// ms, n = 1024 1.61 -> 1.54; at four 0.494 and 1.60).
+template <int S, int NL> __host__ __device__ constexpr int gjw_ctas() {
+  return NL > 28 ? 2 : 512 / (2 * NL + (NL < S ? 2 * S : 0) + 40);
+}
 template <typename C, int S, int NL>
 __global__ void __launch_bounds__(32 * GJW_FRONTS, gjw_ctas<S, NL>()) k_gj_warp(LevelK<C> L, LevelK<C> Ch, int has_child, int* err, int ring) {
   constexpr int G = 32 / S;
