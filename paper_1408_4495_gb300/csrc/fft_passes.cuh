@@ -11,9 +11,10 @@
 // pass (16 store-and-load rounds with two barriers each in the L = 2048 symbol pass, now 4 with
 // one): FP32, 2D n = 512, 16 vectors: rows forward / symbol / rows inverse 53 / 149 / 61 us -> 20
 // / 61 / 25 us; n = 1024, 64 vectors: symbol pass 2.23 -> 1.39 ms; float-float 8.0 -> 5.0 ms.  What
-// bounds them: FP32 the shared-memory path and issue slots (1.4 TB/s through the symbol pass),
-// float-float the FP32 pipe (its additions are 8 packed instructions a complex number, about 160
-// for a point of an L = 2048 transform), FP64 its pipe (1.9 FMAs a clock and SM).
+// bounds them (counters at 2D n = 1024, 16 vectors): FP32 the path to L1 and shared memory (79 %
+// busy, 1.4 TB/s through the symbol pass; the row passes 75 and 83 % of the memory bandwidth), float-float
+// the FP32 pipe (81 % active in the symbol pass: 418 instructions a point of the padded grid, additions of 8 packed
+// ones a complex number), FP64 its pipe (85 % active at n = 256).
 #pragma once
 
 #include <atomic>
