@@ -2422,7 +2422,6 @@ template <typename C> struct SweepK {
                      // order by the CTA that finishes last
   int ksz;           // columns per range
   int kv;            // items of the vector operand held in shared memory at once
-  int leaf;          // small levels: 1 where w_own is r_own and stays in T (sweep_leaf)
   int ng;            // groups of RC right-hand sides: the CTAs of one front's groups are
                      // adjacent in the grid (x = front * ng + group), so that its factor tile
                      // is read from DRAM once and from L2 by the other groups
@@ -2885,7 +2884,9 @@ __global__ void __launch_bounds__(256) k_tcs_scatter(SweepK<float2> S, const flo
 // and 0.90 (their bytes at the copy rate: 1.8, 1.2, 0.8, 0.5).  Backward the stores stay with the
 // rows' lanes and the products scalar: packed accumulators and the detour take 72 registers against
 // 48, which cost the leaves 4.70 against 3.36 ms.
-// At the leaves w_own is r_own, which stays in T where both sweeps of the level run here (sweep_leaf).
+// At the leaves w_own is r_own, which stays in T where both sweeps of the level run here (leaf, by
+// sweep_leaf; not a field of SweepK, whose layout k_sweep's register allocation hangs on: with one more field
+// FP64 applications at 3D n = 16 with 64 right-hand sides took 1.80 ms against 1.69).
 constexpr int SMALL_FPC = 4;   // warps per CTA at most (groups of 16 of SOLVE_CHUNK)
 constexpr int SMALL_KCH = 64;  // columns of the factor tile and operand staged at once
 // Fronts from which the updates are gathered ahead of the product: below, the chain of a CTA counts
@@ -2918,7 +2919,7 @@ __device__ __forceinline__ float2 unpack2(unsigned long long v) {
   return r;
 }
 template <int MODE, int RP, bool MULTI>
-__global__ void __launch_bounds__(32 * SMALL_FPC) k_sweep_small(SweepK<float2> S) {
+__global__ void __launch_bounds__(32 * SMALL_FPC) k_sweep_small(SweepK<float2> S, int leaf) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int NRB = RP / 16, NJ = 8;
   constexpr bool PACK = MODE == 0 && NRB == 1;
@@ -2945,7 +2946,7 @@ __global__ void __launch_bounds__(32 * SMALL_FPC) k_sweep_small(SweepK<float2> S
     }
     cp_async_commit();
   };
-  const bool leaf = S.leaf != 0, child = MODE == 0 && S.nf_c > 0;
+  const bool child = MODE == 0 && S.nf_c > 0;
   const bool early = child && S.nf >= SMALL_EARLY_FRONTS;  // the updates are gathered with the operand
   // ---- prologue: static data only
   load_chunk(0);
@@ -3179,7 +3180,7 @@ template <int MODE> static void launch_sweep_small(NdPlan* p, int l, float2* T, 
   S.N = p->N;
   const int K = MODE == 0 ? D.smax : D.bmax + D.smax;
   const int rows = MODE == 0 ? D.bmax : D.smax;
-  S.leaf = sweep_leaf(p, l, ng);
+  const int leaf = sweep_leaf(p, l, ng);
   const int rp = (rows + 15) / 16 * 16;
   const size_t smem = small_smem_bytes(MODE, K, rp, ng);
   // one CTA per front, one warp per group
@@ -3195,7 +3196,7 @@ template <int MODE> static void launch_sweep_small(NdPlan* p, int l, float2* T, 
                                    (int)small_smem_bytes(MODE, SMALL_MAX_K, RP, SMALL_FPC)));
       attr.store(true, std::memory_order_release);
     }
-    LS_LAUNCH(cls, st, launch_pdl(k_sweep_small<MODE, RP, MULTI>, grid, block, smem, st, S));
+    LS_LAUNCH(cls, st, launch_pdl(k_sweep_small<MODE, RP, MULTI>, grid, block, smem, st, S, leaf));
   };
   auto by_chunks = [&](auto rpc) {
     if (multi) launch(rpc, std::true_type());
